@@ -19,10 +19,10 @@ struct SeqState {             // device state of the batch (all [batch] unless n
   int32_t* ctx_len;
   int32_t* nvalid;            // tree nodes scored for the sequence this iteration (0: inactive)
   int32_t* gen_count;         // tokens generated so far
-  int32_t* commit_base;       // context length before the commit
-  int32_t* commit_len;        // accepted length
-  int32_t* commit_path;       // [batch][kMaxPath] node ids of the winning path
-  int32_t* best;              // winning node
+  int32_t* commit_base;       // ctx_len as the acceptance saw it: the commit's blocks read this while one of them moves ctx_len on
+  int32_t* commit_nv;         // the same of nvalid
+  int32_t* node_ok;           // [batch][kMaxNodes]: the node is among its parent's draws
+  int32_t* node_top;          // [batch][kMaxNodes]: the node's first draw, where accept_kernel forms it
   int32_t* out_tokens;        // [batch][out_cap] generated tokens (may be null)
   int32_t* done_count;        // scalar: sequences that reached the target
   int out_cap;
@@ -30,33 +30,117 @@ struct SeqState {             // device state of the batch (all [batch] unless n
   unsigned long long* stats;  // [2][kStatDepth][kStatTopk]: acceptance tests applied / passed, by (draft head, rank)
 };
 
+// (a grid of more than two blocks of 512 per SM is bound by throughput: smaller blocks, fewer barriers' worth of idling)
+inline int accept_threads(int vocab, int blocks) { return vocab > kSelectWide ? 1024 : blocks <= 4 * 148 ? 512 : 256; }
 
-// One block per sequence.  A sequence whose path commits EOS (when EOS is not masked) or reaches the token
-// target becomes inactive (nvalid = 0).  Edges are tested depth by depth, only below accepted nodes:
-// for an accepted parent p the keys of its logits row are formed once in shared memory
-// (they predict absolute position ctx_len + depth(p) + 1), then each child token c is
-// accepted iff fewer than tau tokens precede it in key order (and it lies in the nucleus).
-// dynamic shared memory: 2 * ld floats.
-__global__ void __launch_bounds__(256) accept_kernel(
-    const float* __restrict__ logits, int ld, int vocab, const int32_t* __restrict__ tokens, TreeView tree,
-    const int32_t* __restrict__ block_table, KvGeom geom, SamplingDev sp,
-    const int32_t* __restrict__ forced_best, SeqState st, AcceptOut out, uint32_t* err) {
-  extern __shared__ float keys[];          // [ld] keys, then [ld] probabilities (nucleus only)
-  float* probs = keys + ld;
-  __shared__ int s_parent[kMaxNodes], s_depth[kMaxNodes], s_tok[kMaxNodes];
-  __shared__ int s_child[kMaxNodes], s_ok[kMaxNodes], s_nchild;
-  __shared__ unsigned long long s_edges[2], s_acc[2];    // bits 0..63, 64..127
-  __shared__ int s_path[kMaxPath], s_best, s_len, s_eos;
-  __shared__ int s_first[kMaxPath + 2];    // nodes are ordered by depth: first node of every depth, then nv
-  __shared__ Best bscratch[32];
-  __shared__ float fscratch[32];
-  __shared__ int s_scan[256];
+// grid = (most inner nodes of a tree, batch): one block per node that has children; or (nodes, batch) with inner = null: a
+// block per node, which then also leaves the node's first draw (the token that continues the sequence if it wins).  The draws of every such node are
+// formed at once, whether or not it turns out to be accepted (the keys of its logits row predict absolute position
+// ctx_len + depth + 1): child token c is accepted iff fewer than tau tokens precede it in key order (and it lies in the
+// nucleus).  commit_kernel walks the tree.  Bound by latency: one block per sequence that formed the keys of one
+// accepted parent after another and walked the tree took 18-26 us at 1025 tokens (three or four parents, 16 block barriers
+// each), 178 us with the nucleus at 2049, 945 us at 16001.  Few tokens per thread (the two logarithms of a token's noise
+// are a chain of 400 cycles) and short code (it runs once per block, from a cold instruction cache) matter more than the
+// operations.  The noise is formed, and everything but the logits is read, while the product that makes the logits still
+// runs: that product waits for its own predecessors before it lets this kernel start.
+// Dynamic shared memory: row_keys_smem.  accept_threads(vocab) threads.
+__global__ void __launch_bounds__(1024) accept_kernel(
+    const float* __restrict__ logits, int ld, int vocab, const int32_t* tokens, TreeView tree,
+    const int32_t* __restrict__ inner /*[kMaxNodes] per tree, -1 behind the last; or null*/, SamplingDev sp, SeqState st) {
+  extern __shared__ float keys[];          // [ld] keys, then [ld] logits (nucleus only)
+  __shared__ SelectScratch sc;
+  __shared__ int s_node[kMaxNodes], s_tok[kMaxNodes], s_cnt[kMaxNodes], s_n, s_depth;
+  const int b = blockIdx.y, N = tree.n_nodes, tid = threadIdx.x, lane = tid & 31;
+  const int to = tree.off(b);
+  // (L2 loads: these were written by kernels before the one that may still be running)
+  const int nv = __ldcg(st.nvalid + b), S = __ldcg(st.ctx_len + b);
+  const int p = inner ? inner[(tree.per_seq ? b * kMaxNodes : 0) + blockIdx.x] : (int)blockIdx.x;
+  int par = -1, tok = 0, dep = 0;
+  if (tid < N) {
+    par = tree.parent[to + tid]; dep = tree.depth[to + tid];
+    tok = __ldcg(tokens + (long long)b * N + tid);
+  }
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+  const bool live = p >= 0 && p < nv;
+  if (live && tid < nv) {
+    if (tid == p) s_depth = dep;
+    if (par == p) { const int i = atomicAdd(&s_n, 1); s_node[i] = tid; s_tok[i] = tok; s_cnt[i] = 0; }
+  }
+  __syncthreads();
+  const uint64_t rs = noise_row_state(sp.seed, b, S + s_depth + 1);
+  if (live && sp.accept_rule == 0) row_noise(vocab, rs, sp, keys);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blockIdx.x == 0 && tid == 0) { st.commit_base[b] = S; st.commit_nv[b] = nv; }
+  if (!live) return;
+  row_keys(base_row(logits + ((long long)b * N + p) * ld, sp, b), vocab, rs, sp, sp.accept_rule == 0, keys, keys + ld, sc);
+  const int nchild = s_n;
+#pragma unroll 1
+  for (int i = 0; i < nchild; ++i) {
+    const int c = s_tok[i];
+    if (c < 0 || c >= vocab) continue;     // not a speech token: never accepted
+    const float kc = keys[c];
+    int cnt = 0;
+#pragma unroll 4
+    for (int j = tid; j < vocab; j += blockDim.x) cnt += precedes(keys[j], j, kc, c) ? 1 : 0;
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0 && cnt) atomicAdd(&s_cnt[i], cnt);
+  }
+  __syncthreads();
+  if (tid < nchild) {
+    const int c = s_tok[tid];
+    st.node_ok[b * kMaxNodes + s_node[tid]] = c >= 0 && c < vocab && s_cnt[tid] < sp.tau && keys[c] > -INFINITY ? 1 : 0;
+  }
+  if (!inner) {
+    const int first = first_key(keys, vocab, sc);
+    if (tid == 0) st.node_top[b * kMaxNodes + p] = first;
+  }
+}
 
-  const int b = blockIdx.x, N = tree.n_nodes, nv = st.nvalid[b];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// floats of the carried logits that one block of commit_kernel copies
+constexpr int kCommitLogits = 4096;
+
+// grid = (n_layers + ceil(ld / kCommitLogits) + 1, batch).  Every block finds the winner for itself: a node is accepted
+// iff it and all its ancestors are among their parents' draws (one mask test per node), the deepest accepted node wins,
+// the smallest index among equally deep ones.  Then
+//   x < n_layers: move the K/V rows of the winning path of layer x from slot base + path[j] to slot base + j, 16 bytes per
+//     thread and step; a thread always handles the same 16-byte column of every row, and rows are read in ascending j
+//     no later than they are overwritten;
+//   the next blocks: carry the winner's hidden state and logits, 16 bytes per thread and step;
+//   the last: outputs, statistics, the sequence's new state.  A sequence whose path commits EOS (when EOS is not
+//     masked) or reaches the token target becomes inactive (nvalid = 0).
+// next_root: accept_kernel has left it with the node (have_top), or the last block draws it here.
+// Dynamic shared memory: row_keys_smem if it has to draw, else none.
+template <typename T>
+__global__ void __launch_bounds__(1024) commit_kernel(
+    T* __restrict__ pool, KvGeom geom, const int32_t* __restrict__ block_table, SeqState st, int n_layers, TreeView tree,
+    const int32_t* tokens, SamplingDev sp, const int32_t* __restrict__ forced_best, int have_top, AcceptOut out,
+    const T* __restrict__ hfinal, int d_model, const float* __restrict__ logits, int ld, int vocab,
+    T* __restrict__ hstar, float* __restrict__ logits_star, uint32_t* err) {
+  extern __shared__ float keys[];
+  __shared__ unsigned long long s_anc[kMaxNodes][2];
+  __shared__ int s_depth[kMaxNodes], s_path[kMaxPath], s_top[kMaxNodes / 32], s_end;
+  __shared__ uint32_t s_edge[kMaxNodes / 32], s_acc[kMaxNodes / 32];
+  const int b = blockIdx.y, N = tree.n_nodes, tid = threadIdx.x, warp = tid >> 5;
+  const int to = tree.off(b);
+  int par = -1, dep = 0, tok = -1;
+  unsigned long long a0 = ~0ull, a1 = ~0ull;
+  if (tid < N) {
+    par = tree.parent[to + tid]; dep = tree.depth[to + tid];
+    tree.anc_of(b, tid, a0, a1);
+    tok = __ldcg(tokens + (long long)b * N + tid);     // (written before the product of the vocabulary head)
+    s_anc[tid][0] = a0; s_anc[tid][1] = a1;
+    s_depth[tid] = dep;
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int nv = st.commit_nv[b], S = st.commit_base[b];
+  const int fb = forced_best ? forced_best[b] : -1;
+  const bool ok = tid == 0 || (tid < N && par >= 0 && st.node_ok[b * kMaxNodes + tid] != 0);
+  const int nlog = (ld + kCommitLogits - 1) / kCommitLogits, part = (int)blockIdx.x - n_layers;
   if (nv == 0) {
+    if (part != nlog) return;
     if (tid == 0) {
-      st.commit_len[b] = 0;
       if (out.accept_len) out.accept_len[b] = 0;
       if (out.edge_bits) for (int w = 0; w < (int)out.edge_words; ++w) out.edge_bits[b * out.edge_words + w] = 0ull;
       if (out.next_root) out.next_root[b] = -1;
@@ -68,203 +152,112 @@ __global__ void __launch_bounds__(256) accept_kernel(
     }
     return;
   }
-  const int S = st.ctx_len[b];
-  const int to = tree.off(b);
+  const bool forced = fb >= 0 && fb < nv;
   if (tid < kMaxNodes) {
-    const bool in = tid < nv;
-    s_parent[tid] = in ? tree.parent[to + tid] : -1;
-    s_depth[tid] = in ? tree.depth[to + tid] : -1;
-    s_tok[tid] = in ? tokens[(long long)b * N + tid] : -1;
+    const uint32_t e = __ballot_sync(0xffffffffu, ok && tid < nv);
+    if ((tid & 31) == 0) s_edge[warp] = e;
   }
-  if (tid == 0) { s_edges[0] = 1ull; s_acc[0] = 1ull; s_edges[1] = 0ull; s_acc[1] = 0ull; }
-  if (tid < kMaxPath + 2) s_first[tid] = nv;
+  if (tid == 0) s_end = kMaxPath;
   __syncthreads();
-  if (tid < nv && (tid == 0 || s_depth[tid] != s_depth[tid - 1])) s_first[min(s_depth[tid], kMaxPath)] = tid;
-  __syncthreads();
-  const int maxdepth = min(s_depth[nv - 1], kMaxPath - 1);
-  const bool nuc = nucleus_on(sp);
-  const int fb = forced_best ? forced_best[b] : -1;
-
-  for (int d = 0; d < maxdepth && fb < 0; ++d) {
-    __syncthreads();                               // the accepted set of depth d is final
-    const unsigned long long a0 = s_acc[0], a1 = s_acc[1];
-    const int p_end = s_first[d + 1];
-    bool any = false;
-    for (int p = s_first[d]; p < p_end; ++p) {
-      if (!bit_at(a0, a1, p)) continue;            // uniform
-      any = true;
-      __syncthreads();
-      if (tid == 0) s_nchild = 0;
-      __syncthreads();
-      if (tid < nv && s_parent[tid] == p) s_child[atomicAdd(&s_nchild, 1)] = tid;
-      __syncthreads();
-      const int nchild = s_nchild;
-      if (nchild == 0) continue;
-      const BaseRow row = base_row(logits + ((long long)b * N + p) * ld, sp, b);
-      const uint64_t rs = noise_row_state(sp.seed, b, S + d + 1);
-      const bool noise = sp.accept_rule == 0;
-      for (int j = tid; j < vocab; j += blockDim.x) keys[j] = key_of(row[j], j, rs, sp, noise);
-      if (nuc) {
-        // Tokens outside the top-p nucleus cannot be drawn: give them the key -inf.  In the order "larger logit,
-        // then lower id" the nucleus is the prefix of tokens whose mass ahead of them is below top_p.  The mass
-        // strictly above a logit value falls as the value grows, so the smallest value v* whose mass above is
-        // still below top_p is found by bisection on the ordered bit pattern of the value (32 block-wide sums
-        // instead of one pass per token); tokens above v* are inside, tokens below it outside, and the tokens
-        // AT v* (equal logits, equal probability p*) are inside while (mass above v*) + (ties with a lower
-        // id) * p* stays below top_p.  probs[] holds exp((l - max) / T).
-        const RowStats rst = row_stats(row, vocab, sp, fscratch);
-        for (int j = tid; j < vocab; j += blockDim.x)
-          probs[j] = expf((masked_logit(row[j], j, sp) - rst.maxl) * sp.inv_temperature);
-        __syncthreads();
-        const float limit = sp.top_p * rst.z;
-        auto mass_above = [&](uint32_t k) -> float {              // sum of p over tokens whose value orders above k
-          float m = 0.f;
-          for (int j = tid; j < vocab; j += blockDim.x)
-            if (ordered_bits(masked_logit(row[j], j, sp)) > k) m += probs[j];
-          return block_sum(m, fscratch);
-        };
-        uint32_t lo = 0u, hi = 0xffffffffu;                       // mass_above(hi) = 0 < limit: v* in (lo, hi]
-        if (mass_above(0u) < limit) hi = 0u;                      // (everything is inside)
-        while (hi - lo > 1u) {
-          const uint32_t mid = lo + ((hi - lo) >> 1);
-          if (mass_above(mid) < limit) hi = mid; else lo = mid;
-        }
-        const float above = mass_above(hi);
-        // ties at v*: exclusive count of earlier ids with the same value, by contiguous chunks of ids
-        const int chunk = (vocab + (int)blockDim.x - 1) / (int)blockDim.x, j0 = tid * chunk, j1 = min(vocab, j0 + chunk);
-        int mine = 0;
-        for (int j = j0; j < j1; ++j) mine += ordered_bits(masked_logit(row[j], j, sp)) == hi ? 1 : 0;
-        __syncthreads();
-        s_scan[tid] = mine;
-        __syncthreads();
-        int before = 0;
-        for (int t = 0; t < tid; ++t) before += s_scan[t];
-        for (int j = j0; j < j1; ++j) {
-          const uint32_t kj = ordered_bits(masked_logit(row[j], j, sp));
-          bool inside = kj > hi;
-          if (kj == hi) { inside = above + (float)before * probs[j] < limit; ++before; }
-          if (!inside) keys[j] = -INFINITY;
-        }
-      }
-      __syncthreads();
-      for (int i = warp; i < nchild; i += (blockDim.x >> 5)) {
-        const int c = s_tok[s_child[i]];
-        int cnt = sp.tau;                                            // not a speech token: never accepted
-        bool finite = false;
-        if (c >= 0 && c < vocab) {
-          const float kc = keys[c];
-          finite = kc > -INFINITY;
-          cnt = 0;
-          for (int j = lane; j < vocab; j += 32) cnt += precedes(keys[j], j, kc, c) ? 1 : 0;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        }
-        if (lane == 0) s_ok[i] = (cnt < sp.tau && finite) ? 1 : 0;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        for (int i = 0; i < nchild; ++i)
-          if (s_ok[i]) { const int c = s_child[i]; s_edges[c >> 6] |= 1ull << (c & 63); s_acc[c >> 6] |= 1ull << (c & 63); }
-      }
-      if (tid < nchild && st.stats && d < kStatDepth) {
-        const int r = tree.rank[to + s_child[tid]];
-        if (r >= 0 && r < kStatTopk) {
-          atomicAdd(st.stats + d * kStatTopk + r, 1ull);
-          if (s_ok[tid]) atomicAdd(st.stats + (kStatDepth + d) * kStatTopk + r, 1ull);
-        }
-      }
-      __syncthreads();
-    }
-    if (!any) break;                               // nothing accepted at this depth: nothing below it either
+  bool acc = false;
+  if (tid < kMaxNodes) {
+    const unsigned long long e0 = s_edge[0] | ((unsigned long long)s_edge[1] << 32), e1 = s_edge[2] | ((unsigned long long)s_edge[3] << 32);
+    acc = tid < nv && (fb < 0 ? ((a0 & ~e0) | (a1 & ~e1)) == 0ull : tid == 0);
+    const uint32_t w = __ballot_sync(0xffffffffu, acc);
+    // deepest first, then the smallest index
+    const int top = __reduce_max_sync(0xffffffffu, acc ? (dep << 8) | (255 - tid) : 0);
+    if ((tid & 31) == 0) { s_acc[warp] = w; s_top[warp] = top; }
   }
   __syncthreads();
-  if (tid == 0) {
-    int best = 0;
-    if (fb >= 0 && fb < nv) best = fb;
-    else {
-      // deepest accepted node, the first (leftmost) of that depth
-      const unsigned long long a0 = s_acc[0], a1 = s_acc[1];
-      for (int d = maxdepth; d >= 1 && best == 0; --d)
-        for (int n = s_first[d]; n < s_first[d + 1]; ++n)
-          if (bit_at(a0, a1, n)) { best = n; break; }
-    }
-    int len = min(s_depth[best] + 1, kMaxPath);
-    int n = best;
-    for (int j = len - 1; j >= 0; --j) { s_path[j] = n; n = s_parent[n]; }
+  int best = forced ? fb : 255 - (max(max(s_top[0], s_top[1]), max(s_top[2], s_top[3])) & 255);
+  // the path is the winner's ancestors, a node per depth
+  const bool on = tid < nv && bit_at(s_anc[best][0], s_anc[best][1], tid) && dep < kMaxPath;
+  if (on) {
+    s_path[dep] = tid;
     // EOS not masked: the sequence ends with the first EOS on the path; what follows it is dropped
-    s_eos = 0;
-    if (!sp.eos_masked)
-      for (int j = 0; j < len; ++j)
-        if (s_tok[s_path[j]] == sp.eos_id) { len = j + 1; best = s_path[j]; s_eos = 1; break; }
-    s_best = best; s_len = len;
+    if (!sp.eos_masked && tok == sp.eos_id) atomicMin(&s_end, dep);
   }
+  int len = min(s_depth[best] + 1, kMaxPath);
   __syncthreads();
-  const int best = s_best, len = s_len;
-  const int nroot = sample_row(base_row(logits + ((long long)b * N + best) * ld, sp, b), vocab, b, S + len, sp, bscratch, fscratch);
+  const bool eos = s_end < len;
+  if (eos) { len = s_end + 1; best = s_path[s_end]; }
 
-  if (tid < kMaxPath) {
-    const bool in = tid < len;
-    const int node = in ? s_path[tid] : -1;
-    st.commit_path[b * kMaxPath + tid] = node;
-    long long slot = -1;
-    if (in) {
-      const long long blk = kv_block_of(block_table, geom, b, S + tid, err);
-      slot = blk < 0 ? -1 : blk * kKvBlock + (S + tid) % kKvBlock;
-    }
-    if (out.path_nodes) out.path_nodes[b * kMaxPath + tid] = node;
-    if (out.path_tokens) out.path_tokens[b * kMaxPath + tid] = in ? s_tok[node] : -1;
-    if (out.kv_slots) out.kv_slots[b * kMaxPath + tid] = slot;
-    if (in && st.out_tokens) {
-      const int g = st.gen_count[b] + tid;
-      if (g < st.out_cap) st.out_tokens[(long long)b * st.out_cap + g] = s_tok[node];
-    }
+  if (part >= 0 && part < nlog) {
+    const long long m = (long long)b * N + best;
+    // (d_model and ld are multiples of 64 and 128: whole 16-byte pieces)
+    const uint4* hs = reinterpret_cast<const uint4*>(hfinal + m * d_model);
+    uint4* hd = reinterpret_cast<uint4*>(hstar + (long long)b * d_model);
+    if (part == 0)
+      for (int i = tid; i < d_model * (int)sizeof(T) / 16; i += blockDim.x) hd[i] = hs[i];
+    const uint4* ls = reinterpret_cast<const uint4*>(logits + m * ld);
+    uint4* l = reinterpret_cast<uint4*>(logits_star + (long long)b * ld);
+    const int end = min(ld, (part + 1) * kCommitLogits) / 4;
+#pragma unroll 4
+    for (int i = part * (kCommitLogits / 4) + tid; i < end; i += blockDim.x) l[i] = ls[i];
+    return;
   }
-  __syncthreads();
-  if (tid == 0) {
-    st.commit_base[b] = S;
-    st.commit_len[b] = len;
-    st.best[b] = best;
-    st.ctx_len[b] = S + len;
-    const int g = st.gen_count[b] + len;
-    st.gen_count[b] = g;
-    if (s_eos || (st.target > 0 && g >= st.target)) { st.nvalid[b] = 0; atomicAdd(st.done_count, 1); }
-    if (out.accept_len) out.accept_len[b] = len;
-    if (out.edge_bits) for (int w = 0; w < (int)out.edge_words; ++w) out.edge_bits[b * out.edge_words + w] = s_edges[w];
-    if (out.next_root) out.next_root[b] = nroot;
-  }
-}
-
-// grid = (n_layers + 1, batch).  x < n_layers: move the K/V rows of the winning path of
-// layer x from slot base + path[j] to slot base + j, 16 bytes per thread and step; a
-// thread always handles the same 16-byte column of every row, and rows are taken in
-// ascending j, so a destination is never read again after it was overwritten.
-// x == n_layers: carry the winner's hidden state and logits.
-template <typename T>
-__global__ void __launch_bounds__(256) commit_kernel(
-    T* __restrict__ pool, KvGeom geom, const int32_t* __restrict__ block_table, SeqState st,
-    int n_layers, int n_nodes, const T* __restrict__ hfinal, int d_model, const float* __restrict__ logits, int ld,
-    T* __restrict__ hstar, float* __restrict__ logits_star, uint32_t* err) {
-  const int b = blockIdx.y, len = st.commit_len[b];
-  if (len == 0) return;
-  if ((int)blockIdx.x == n_layers) {
-    const long long m = (long long)b * n_nodes + st.best[b];
-    for (int i = threadIdx.x; i < d_model; i += blockDim.x) hstar[(long long)b * d_model + i] = hfinal[m * d_model + i];
-    for (int i = threadIdx.x; i < ld; i += blockDim.x) logits_star[(long long)b * ld + i] = logits[m * ld + i];
+  if (part == nlog) {
+    int g = 0;
+    if (st.out_tokens || tid == 0) g = st.gen_count[b];
+    if (tid < kMaxPath) {
+      const bool in = tid < len;
+      if (out.path_nodes) out.path_nodes[b * kMaxPath + tid] = in ? s_path[tid] : -1;
+      if (out.kv_slots) {
+        long long slot = -1;
+        if (in) {
+          const long long blk = kv_block_of(block_table, geom, b, S + tid, err);
+          slot = blk < 0 ? -1 : blk * kKvBlock + (S + tid) % kKvBlock;
+        }
+        out.kv_slots[b * kMaxPath + tid] = slot;
+      }
+      if (out.path_tokens && !in) out.path_tokens[b * kMaxPath + tid] = -1;
+    }
+    if (on && dep < len) {
+      if (out.path_tokens) out.path_tokens[b * kMaxPath + dep] = tok;
+      if (st.out_tokens && g + dep < st.out_cap) st.out_tokens[(long long)b * st.out_cap + g + dep] = tok;
+    }
+    // tests applied and passed, by (draft head, rank)
+    if (st.stats && fb < 0 && tid < nv && par >= 0 && ((s_acc[par >> 5] >> (par & 31)) & 1u)) {
+      const int d = dep - 1, r = tree.rank[to + tid];
+      if (d < kStatDepth && r >= 0 && r < kStatTopk) {
+        atomicAdd(st.stats + d * kStatTopk + r, 1ull);
+        if (acc) atomicAdd(st.stats + (kStatDepth + d) * kStatTopk + r, 1ull);
+      }
+    }
+    __syncthreads();                             // (every thread has read gen_count)
+    if (tid == 0) {
+      st.ctx_len[b] = S + len;
+      st.gen_count[b] = g + len;
+      if (eos || (st.target > 0 && g + len >= st.target)) { st.nvalid[b] = 0; atomicAdd(st.done_count, 1); }
+      if (out.accept_len) out.accept_len[b] = len;
+      if (out.edge_bits)
+        for (int w = 0; w < (int)out.edge_words; ++w)
+          out.edge_bits[b * out.edge_words + w] = s_acc[2 * w] | ((unsigned long long)s_acc[2 * w + 1] << 32);
+    }
+    if (out.next_root && have_top) {
+      if (tid == 0) out.next_root[b] = st.node_top[b * kMaxNodes + best];
+    } else if (out.next_root) {
+      __shared__ SelectScratch sc;
+      const uint64_t rs = noise_row_state(sp.seed, b, S + len);
+      row_noise(vocab, rs, sp, keys);
+      row_keys(base_row(logits + ((long long)b * N + best) * ld, sp, b), vocab, rs, sp, true, keys, keys + ld, sc);
+      const int next = first_key(keys, vocab, sc);
+      if (tid == 0) out.next_root[b] = next;
+    }
     return;
   }
   __shared__ long long s_src[kMaxPath], s_dst[kMaxPath];
-  const int base = st.commit_base[b];
-  if (threadIdx.x < kMaxPath) {
-    const int j = threadIdx.x;
+  if (tid < kMaxPath) {
+    const int j = tid;
     long long src = -1, dst = -1;
     if (j < len) {
-      const int node = st.commit_path[b * kMaxPath + j];
+      const int node = s_path[j];
       if (node != j) {
-        const long long bs = kv_block_of(block_table, geom, b, base + node, err);
-        const long long bd = kv_block_of(block_table, geom, b, base + j, err);
+        const long long bs = kv_block_of(block_table, geom, b, S + node, err);
+        const long long bd = kv_block_of(block_table, geom, b, S + j, err);
         if (bs >= 0 && bd >= 0) {
-          src = geom.elem(bs, 0, 0, (base + node) % kKvBlock);
-          dst = geom.elem(bd, 0, 0, (base + j) % kKvBlock);
+          src = geom.elem(bs, 0, 0, (S + node) % kKvBlock);
+          dst = geom.elem(bd, 0, 0, (S + j) % kKvBlock);
         }
       }
     }
@@ -275,13 +268,16 @@ __global__ void __launch_bounds__(256) commit_kernel(
   const int cpr = geom.head_dim * (int)sizeof(T) / 16;            // 16-byte chunks per row
   const int chunks = 2 * geom.n_heads * cpr;
   const long long row_stride = (long long)kKvBlock * geom.head_dim;   // elements between (kv, head) tiles
-  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
+  for (int c = tid; c < chunks; c += blockDim.x) {
     const int tile = c / cpr, cc = c % cpr;
-    for (int j = 1; j < len; ++j) {
-      if (s_src[j] < 0) continue;
-      const uint4* s = reinterpret_cast<const uint4*>(lp + s_src[j] + tile * row_stride) + cc;
-      uint4* dd = reinterpret_cast<uint4*>(lp + s_dst[j] + tile * row_stride) + cc;
-      *dd = *s;
+    for (int j0 = 1; j0 < len; j0 += 4) {                         // four rows in flight
+      uint4 v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (j0 + i < len && s_src[j0 + i] >= 0) v[i] = *(reinterpret_cast<const uint4*>(lp + s_src[j0 + i] + tile * row_stride) + cc);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (j0 + i < len && s_src[j0 + i] >= 0) *(reinterpret_cast<uint4*>(lp + s_dst[j0 + i] + tile * row_stride) + cc) = v[i];
     }
   }
 }

@@ -50,6 +50,7 @@ struct vadusa_ctx {
   int tree_per_seq = 0;
   int max_rank_used = 0;
   int tree_max_depth = 0;
+  int tree_inner = 0;         // most nodes with children of any of the trees
   // draft-head fitting (vadusa_fit_*): the caller's state buffer and the schedule
   char* fit = nullptr;
   int fit_tokens = 0, fit_step = 0, fit_warmup = 0;
@@ -197,9 +198,9 @@ SeqState state_of(vadusa_ctx* c, int32_t* out_tokens, int out_cap, int target) {
   s.nvalid = wsptr<int32_t>(c, c->ws.nvalid);
   s.gen_count = wsptr<int32_t>(c, c->ws.gen_count);
   s.commit_base = wsptr<int32_t>(c, c->ws.commit_base);
-  s.commit_len = wsptr<int32_t>(c, c->ws.commit_len);
-  s.commit_path = wsptr<int32_t>(c, c->ws.commit_path);
-  s.best = wsptr<int32_t>(c, c->ws.best);
+  s.commit_nv = wsptr<int32_t>(c, c->ws.commit_nv);
+  s.node_ok = wsptr<int32_t>(c, c->ws.node_ok);
+  s.node_top = wsptr<int32_t>(c, c->ws.node_top);
   s.out_tokens = out_tokens;
   s.done_count = done_word(c);
   s.out_cap = out_cap;
@@ -227,6 +228,21 @@ vadusa_status sampling_dev(vadusa_ctx* ctx, const vadusa_sampling* s, SamplingDe
   o->bias = ctx->logit_bias;
   o->bias_ld = ctx->logit_bias_ld;
   return VADUSA_OK;
+}
+
+// Launch of a kernel that begins with griddepcontrol.wait: it may be set up while its predecessor is still running.
+template <typename K, typename... A>
+cudaError_t launch_dependent(vadusa_ctx* ctx, K kernel, dim3 grid, int threads, size_t smem, A... args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = ctx->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at; lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, args...);
 }
 
 // ---- typed engine ------------------------------------------------------------------
@@ -470,7 +486,7 @@ bool ln_product(vadusa_ctx* ctx, int cls, const float* x, const float* g, const 
 // pages leave SMs to the next kernel's early CTAs and their weight loads, 128 CTAs of one or two pages do not;
 // 0.538 -> 0.528 ms per step).  The estimate of the context is the host's lower one: never behind by more than
 // the tokens accepted beyond one per iteration since the last exact value.
-// (Ragged batches are balanced by visiting the sequences longest first, see seq_order_kernel.)
+// (Ragged batches are balanced by visiting the sequences longest first, see tree_embed_kernel.)
 constexpr long long kAttLongContext = 1536;
 int attention_splits(const vadusa_ctx* ctx, int n_nodes) {
   int splits = 1;
@@ -718,6 +734,24 @@ vadusa_status fused_forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* 
   return VADUSA_OK;
 }
 
+// Tokens and embeddings of all tree nodes, and the order in which attention visits the sequences.
+template <typename T>
+vadusa_status embed(vadusa_ctx* ctx, const TreeView& tv, const int32_t* override_tokens, long long* kv_row, float2* stats) {
+  const vadusa_config& c = ctx->cfg;
+  const int M = ctx->batch * tv.n_nodes;
+  const bool ordered = ctx->batch > 1;
+  PROF(ctx, K_EMBED);
+  CU(launch_dependent(ctx, tree_embed_kernel<T>, dim3(M + (ordered ? 1 : 0)), 128, 0, tv, override_tokens,
+                      (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.root), (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.topk),
+                      c.n_draft_heads, c.draft_topk, (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.ctx_len),
+                      (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.nvalid), as<T>(ctx->emb_audio), as<T>(ctx->emb_phon),
+                      as<T>(ctx->pos), c.vocab, c.n_phonemes, c.max_pos, c.d_model, wsptr<int32_t>(ctx, ctx->ws.tokens),
+                      wsptr<float>(ctx, ctx->ws.x), ctx->block_table, geom_of(ctx), kv_row, stats, M,
+                      ordered ? wsptr<int32_t>(ctx, ctx->ws.seq_order) : (int32_t*)nullptr, err_word(ctx)));
+  LAUNCH_CHECK();
+  return VADUSA_OK;
+}
+
 // One forward pass of the base model over batch * tv.n_nodes rows (verify step).
 template <typename T>
 vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* override_tokens, T* attn_tap) {
@@ -738,8 +772,6 @@ vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* overri
   T* mid = wsptr<T>(ctx, ctx->ws.mid);
   T* hfinal = wsptr<T>(ctx, ctx->ws.hfinal);
   float* logits = wsptr<float>(ctx, ctx->ws.logits);
-  int32_t* ctx_len = wsptr<int32_t>(ctx, ctx->ws.ctx_len);
-  int32_t* nvalid = wsptr<int32_t>(ctx, ctx->ws.nvalid);
 
   // LayerNorm statistics for the products that normalise their own operand (bf16 models, few tokens): left by
   // the embedding kernel and by the residual products
@@ -747,18 +779,7 @@ vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* overri
   const bool embed_stats = tc && M <= 64 && d % 128 == 0 && d / 128 <= 8;
   const bool stats_out = tc && residual_leaves_stats(M, d, d), stats_ffn = tc && residual_leaves_stats(M, d, f);
   float2* stats = wsptr<float2>(ctx, ctx->ws.ln_stats);
-  PROF(ctx, K_EMBED);
-  tree_embed_kernel<T><<<M, 128, 0, ctx->stream>>>(
-      tv, override_tokens, wsptr<int32_t>(ctx, ctx->ws.root), wsptr<int32_t>(ctx, ctx->ws.topk), c.n_draft_heads,
-      c.draft_topk, ctx_len, nvalid, as<T>(ctx->emb_audio), as<T>(ctx->emb_phon), as<T>(ctx->pos),
-      c.vocab, c.n_phonemes, c.max_pos, d, wsptr<int32_t>(ctx, ctx->ws.tokens), x, ctx->block_table, g,
-      wsptr<long long>(ctx, ctx->ws.kv_row), embed_stats ? stats : nullptr, err_word(ctx));
-  LAUNCH_CHECK();
-  if (B > 1) {
-    PROF(ctx, K_MISC);
-    seq_order_kernel<<<1, 256, 0, ctx->stream>>>(ctx_len, nvalid, B, wsptr<int32_t>(ctx, ctx->ws.seq_order));
-    LAUNCH_CHECK();
-  }
+  if (vadusa_status s = embed<T>(ctx, tv, override_tokens, wsptr<long long>(ctx, ctx->ws.kv_row), embed_stats ? stats : nullptr)) return s;
   bool have_stats = embed_stats;
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerW& w = ctx->layers[l];
@@ -829,11 +850,10 @@ vadusa_status draft(vadusa_ctx* ctx, const SamplingDev& sp) {
   if (s) return s;
   dim3 grid(hd + 1, B);
   PROF(ctx, K_DRAFT_SELECT);
-  draft_select_kernel<<<grid, 256, 0, ctx->stream>>>(dl, wsptr<float>(ctx, ctx->ws.logits_star), vp, c.vocab, B, hd,
-                                                     c.draft_topk, wsptr<int32_t>(ctx, ctx->ws.ctx_len),
-                                                     wsptr<int32_t>(ctx, ctx->ws.nvalid), sp,
-                                                     wsptr<int32_t>(ctx, ctx->ws.topk),
-                                                     wsptr<int32_t>(ctx, ctx->ws.root));
+  CU(launch_dependent(ctx, draft_select_kernel, grid, select_threads(c.vocab), row_keys_smem(vp, sp), (const float*)dl,
+                      (const float*)wsptr<float>(ctx, ctx->ws.logits_star), vp, c.vocab, B, hd, c.draft_topk,
+                      (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.ctx_len), (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.nvalid),
+                      sp, wsptr<int32_t>(ctx, ctx->ws.topk), wsptr<int32_t>(ctx, ctx->ws.root)));
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
@@ -848,16 +868,20 @@ vadusa_status accept_commit(vadusa_ctx* ctx, const SamplingDev& sp, const int32_
   const TreeView tv = tree_of(ctx, false);
   SeqState st = state_of(ctx, out_tokens, out_cap, target);
   PROF(ctx, K_ACCEPT);
-  accept_kernel<<<B, 256, 2 * vp * sizeof(float), ctx->stream>>>(
-      wsptr<float>(ctx, ctx->ws.logits), vp, c.vocab, wsptr<int32_t>(ctx, ctx->ws.tokens), tv, ctx->block_table, g,
-      sp, forced, st, out, err_word(ctx));
+  // the next root is wanted and the device holds a block per node at once: every node's first draw along with the rest
+  const bool tops = out.next_root && sp.accept_rule == 0 && tv.n_nodes * B <= 2 * 148;
+  const int draw_smem = out.next_root && !tops ? (int)row_keys_smem(vp, sp) : 0;
+  CU(launch_dependent(ctx, accept_kernel, dim3(tops ? tv.n_nodes : ctx->tree_inner, B), accept_threads(c.vocab, tv.n_nodes * B), row_keys_smem(vp, sp),
+                      (const float*)wsptr<float>(ctx, ctx->ws.logits), vp, c.vocab,
+                      (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.tokens), tv,
+                      (const int32_t*)(tops ? nullptr : wsptr<int32_t>(ctx, ctx->ws.tree_inner)), sp, st));
   LAUNCH_CHECK();
-  dim3 grid(c.n_layers + 1, B);
   PROF(ctx, K_COMMIT);
-  commit_kernel<T><<<grid, 256, 0, ctx->stream>>>(
-      reinterpret_cast<T*>(c.kv_pool), g, ctx->block_table, st, c.n_layers, tv.n_nodes,
-      wsptr<T>(ctx, ctx->ws.hfinal), c.d_model, wsptr<float>(ctx, ctx->ws.logits), vp, wsptr<T>(ctx, ctx->ws.hstar),
-      wsptr<float>(ctx, ctx->ws.logits_star), err_word(ctx));
+  CU(launch_dependent(ctx, commit_kernel<T>, dim3(c.n_layers + (vp + kCommitLogits - 1) / kCommitLogits + 1, B),
+                      draw_smem ? select_threads(c.vocab) : 256, draw_smem, reinterpret_cast<T*>(c.kv_pool), g, ctx->block_table, st,
+                      c.n_layers, tv, (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.tokens), sp, forced, tops ? 1 : 0, out,
+                      (const T*)wsptr<T>(ctx, ctx->ws.hfinal), c.d_model, (const float*)wsptr<float>(ctx, ctx->ws.logits), vp,
+                      c.vocab, wsptr<T>(ctx, ctx->ws.hstar), wsptr<float>(ctx, ctx->ws.logits_star), err_word(ctx)));
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
@@ -1059,9 +1083,13 @@ vadusa_status set_kernel_attributes(vadusa_ctx* ctx) {
   CU(cudaFuncSetAttribute(prefill_attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemBytes));
   CU(cudaFuncSetAttribute(tree_attention_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAsSmemBytes));
   CU(cudaFuncSetAttribute(prefill_attention_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-  // the accept kernel keeps one row of keys and one of probabilities in shared memory.  The limit is an attribute of
+  // the kernels that draw keep one row of keys and one of logits in shared memory.  The limit is an attribute of
   // the function on this device, shared by every context: always the library's largest vocabulary
   CU(cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
+  CU(cudaFuncSetAttribute(accept_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  CU(cudaFuncSetAttribute(commit_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
+  CU(cudaFuncSetAttribute(commit_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
+  CU(cudaFuncSetAttribute(draft_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
   // ask for the largest shared-memory carve-out so that several CTAs fit on an SM
   CU(cudaFuncSetAttribute(tree_attention_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   CU(cudaFuncSetAttribute(tree_attention_stream_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
@@ -1276,7 +1304,8 @@ vadusa_status vadusa_set_tree(vadusa_ctx* ctx, int32_t n_nodes, const int32_t* h
   }
   std::vector<int32_t> depth((size_t)copies * n_nodes);
   std::vector<unsigned long long> anc((size_t)copies * n_nodes * 2);
-  int max_rank = 0, max_depth = 0;
+  std::vector<int32_t> inner((size_t)copies * VADUSA_MAX_TREE_NODES, -1);
+  int max_rank = 0, max_depth = 0, max_inner = 0;
   for (int s = 0; s < copies; ++s) {
     const int32_t* par = h_parent + (size_t)s * n_nodes;
     const int32_t* rnk = h_rank + (size_t)s * n_nodes;
@@ -1305,17 +1334,25 @@ vadusa_status vadusa_set_tree(vadusa_ctx* ctx, int32_t n_nodes, const int32_t* h
       max_rank = rnk[n] > max_rank ? rnk[n] : max_rank;
       max_depth = dep[n] > max_depth ? dep[n] : max_depth;
     }
+    bool has[VADUSA_MAX_TREE_NODES] = {false};
+    for (int n = 1; n < n_nodes; ++n) has[par[n]] = true;
+    int k = 0;
+    for (int n = 0; n < n_nodes; ++n)
+      if (has[n]) inner[(size_t)s * VADUSA_MAX_TREE_NODES + k++] = n;
+    max_inner = k > max_inner ? k : max_inner;
   }
   const size_t n4 = (size_t)copies * n_nodes * sizeof(int32_t);
   CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_parent, h_parent, n4, cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_rank, h_rank, n4, cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_depth, depth.data(), n4, cudaMemcpyHostToDevice, ctx->stream));
+  CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_inner, inner.data(), inner.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_anc, anc.data(), (size_t)copies * n_nodes * 16, cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
   ctx->n_nodes = n_nodes;
   ctx->tree_per_seq = per_sequence ? 1 : 0;
   ctx->max_rank_used = max_rank;
   ctx->tree_max_depth = max_depth;
+  ctx->tree_inner = max_inner > 0 ? max_inner : 1;
   ctx->have_draft = ctx->have_verify = false;
   if (ctx->batch > 0) return set_active(ctx, ctx->n_nodes);
   return VADUSA_OK;
@@ -1391,21 +1428,7 @@ vadusa_status vadusa_draft(vadusa_ctx* ctx, const vadusa_sampling* sampling, int
       // tokens of the tree without a model pass: the embed kernel computes them; run it alone
       const TreeView tv = tree_of(ctx, false);
       const int M = ctx->batch * tv.n_nodes;
-      if (c.dtype == 1)
-        tree_embed_kernel<bf16><<<M, 128, 0, ctx->stream>>>(
-            tv, nullptr, wsptr<int32_t>(ctx, ctx->ws.root), wsptr<int32_t>(ctx, ctx->ws.topk), c.n_draft_heads, c.draft_topk,
-            wsptr<int32_t>(ctx, ctx->ws.ctx_len), wsptr<int32_t>(ctx, ctx->ws.nvalid), as<bf16>(ctx->emb_audio),
-            as<bf16>(ctx->emb_phon), as<bf16>(ctx->pos), c.vocab, c.n_phonemes, c.max_pos, c.d_model,
-            wsptr<int32_t>(ctx, ctx->ws.tokens), wsptr<float>(ctx, ctx->ws.x), ctx->block_table, geom_of(ctx),
-            (long long*)nullptr, (float2*)nullptr, err_word(ctx));
-      else
-        tree_embed_kernel<float><<<M, 128, 0, ctx->stream>>>(
-            tv, nullptr, wsptr<int32_t>(ctx, ctx->ws.root), wsptr<int32_t>(ctx, ctx->ws.topk), c.n_draft_heads, c.draft_topk,
-            wsptr<int32_t>(ctx, ctx->ws.ctx_len), wsptr<int32_t>(ctx, ctx->ws.nvalid), as<float>(ctx->emb_audio),
-            as<float>(ctx->emb_phon), as<float>(ctx->pos), c.vocab, c.n_phonemes, c.max_pos, c.d_model,
-            wsptr<int32_t>(ctx, ctx->ws.tokens), wsptr<float>(ctx, ctx->ws.x), ctx->block_table, geom_of(ctx),
-            (long long*)nullptr, (float2*)nullptr, err_word(ctx));
-      LAUNCH_CHECK();
+      if (vadusa_status s = DISPATCH(embed<float>(ctx, tv, nullptr, nullptr, nullptr), embed<bf16>(ctx, tv, nullptr, nullptr, nullptr))) return s;
       CU(cudaMemcpyAsync(tree_tokens, ctx->wsp + ctx->ws.tokens, (size_t)M * 4, cudaMemcpyDeviceToDevice, ctx->stream));
     }
     return VADUSA_OK;

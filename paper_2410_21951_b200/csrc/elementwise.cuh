@@ -4,12 +4,23 @@
 
 namespace vadusa {
 
-// One block per tree node row m = b * n_nodes + n.
+// Four consecutive table entries as floats.
+template <typename T> __device__ __forceinline__ float4 load4(const T* p);
+template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
+template <> __device__ __forceinline__ float4 load4<bf16>(const bf16* p) {
+  const uint2 v = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xffff0000u));
+}
+
+// One block per tree node row m = b * n_nodes + n, and one more (if order is not null) that ranks the sequences.
 // token = override ? override[m] : (n == 0 ? root[b] : topk[b][depth-1][rank]);
 // position = ctx_len[b] + depth[n]; x[m] = E[token] + P[position] (fp32); kv_row[m] = cache slot of the node.
 // Token ids >= vocab address the phoneme table.
+// order[r] = the sequence with the r-th longest context (ties: lower index first); inactive sequences last.  The
+// attention grid visits sequences in this order, so the longest chains start first and a ragged batch balances.
 template <typename T>
-__global__ void tree_embed_kernel(TreeView tree, const int32_t* __restrict__ override_tokens,
+__global__ void __launch_bounds__(128) tree_embed_kernel(TreeView tree, const int32_t* __restrict__ override_tokens,
                                   const int32_t* __restrict__ root, const int32_t* __restrict__ topk,
                                   int n_draft_heads, int draft_topk,
                                   const int32_t* __restrict__ ctx_len, const int32_t* __restrict__ nvalid,
@@ -17,8 +28,25 @@ __global__ void tree_embed_kernel(TreeView tree, const int32_t* __restrict__ ove
                                   const T* __restrict__ pos_table, int vocab, int n_phonemes, int max_pos, int d,
                                   int32_t* __restrict__ tokens_out, float* __restrict__ x,
                                   const int32_t* __restrict__ block_table, KvGeom geom, long long* __restrict__ kv_row,
-                                  float2* __restrict__ stats /*[rows][d/128] or null*/, uint32_t* err) {
+                                  float2* __restrict__ stats /*[rows][d/128] or null*/, int rows, int32_t* __restrict__ order,
+                                  uint32_t* err) {
   const int m = blockIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (m == rows) {
+    const int batch = rows / tree.n_nodes;
+    for (int b = threadIdx.x; b < batch; b += blockDim.x) {
+      const int lb = nvalid[b] > 0 ? ctx_len[b] : -1;
+      int rank = 0;
+#pragma unroll 8
+      for (int o = 0; o < batch; ++o) {
+        const int lo = nvalid[o] > 0 ? ctx_len[o] : -1;
+        rank += (lo > lb || (lo == lb && o < b)) ? 1 : 0;
+      }
+      order[rank] = b;
+    }
+    return;
+  }
   const int b = m / tree.n_nodes, n = m % tree.n_nodes;
   const int to = tree.off(b);
   const int depth = tree.depth[to + n];
@@ -47,40 +75,22 @@ __global__ void tree_embed_kernel(TreeView tree, const int32_t* __restrict__ ove
     if (kv_row) kv_row[m] = row;
   }
   const T* p = pos_table + (long long)pos * d;
-  if (stats) {
-    // d is a multiple of 128: warp w takes the groups of 128 features w, w + 4, ... (lane l: features 4l .. 4l+3 of
-    // the group) and leaves each group's mean and sum of squared deviations for the LayerNorm folded into the
-    // first product
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nt = d >> 7;
-    for (int gi = warp; gi < nt; gi += (int)(blockDim.x >> 5)) {
-      const int c0 = 128 * gi + 4 * lane;
-      float4 v;
-      v.x = to_f<T>(e[c0]) + to_f<T>(p[c0]);         v.y = to_f<T>(e[c0 + 1]) + to_f<T>(p[c0 + 1]);
-      v.z = to_f<T>(e[c0 + 2]) + to_f<T>(p[c0 + 2]); v.w = to_f<T>(e[c0 + 3]) + to_f<T>(p[c0 + 3]);
-      *reinterpret_cast<float4*>(x + (long long)m * d + c0) = v;
+  // d is a multiple of 64: warp w takes the groups of 128 features w, w + 4, ... (lane l: features 4l .. 4l+3 of
+  // the group) and, where asked, leaves each group's mean and sum of squared deviations for the LayerNorm folded
+  // into the first product (d a multiple of 128 then)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nt = (d + 127) >> 7;
+  for (int gi = warp; gi < nt; gi += (int)(blockDim.x >> 5)) {
+    const int c0 = 128 * gi + 4 * lane;
+    if (c0 >= d) break;
+    const float4 ve = load4<T>(e + c0), vp = load4<T>(p + c0);
+    float4 v = make_float4(ve.x + vp.x, ve.y + vp.y, ve.z + vp.z, ve.w + vp.w);
+    *reinterpret_cast<float4*>(x + (long long)m * d + c0) = v;
+    if (stats) {
       const float mu = warp_sum((v.x + v.y) + (v.z + v.w)) * (1.0f / 128.0f);
       const float d0 = v.x - mu, d1 = v.y - mu, d2 = v.z - mu, d3 = v.w - mu;
       const float q = warp_sum((d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3));
       if (lane == 0) stats[(long long)m * nt + gi] = make_float2(mu, q);
     }
-    return;
-  }
-  for (int i = threadIdx.x; i < d; i += blockDim.x) x[(long long)m * d + i] = to_f<T>(e[i]) + to_f<T>(p[i]);
-}
-
-// order[r] = the sequence with the r-th longest context (ties: lower index first); inactive
-// sequences last.  The attention grid visits sequences in this order, so the longest chains
-// start first and a ragged batch balances over the SMs.  One block.
-__global__ void seq_order_kernel(const int32_t* __restrict__ ctx_len, const int32_t* __restrict__ nvalid, int batch,
-                                 int32_t* __restrict__ order) {
-  for (int b = threadIdx.x; b < batch; b += blockDim.x) {
-    const int lb = nvalid[b] > 0 ? ctx_len[b] : -1;
-    int rank = 0;
-    for (int o = 0; o < batch; ++o) {
-      const int lo = nvalid[o] > 0 ? ctx_len[o] : -1;
-      rank += (lo > lb || (lo == lb && o < b)) ? 1 : 0;
-    }
-    order[rank] = b;
   }
 }
 

@@ -97,10 +97,11 @@ inline std::vector<TensorDesc> weight_layout(const vadusa_config* c, int64_t* to
 
 struct WorkspaceLayout {
   int64_t scalars;                       // uint32 err, int32 done_count, padding
-  int64_t ctx_len, nvalid, gen_count, commit_base, commit_len, best, root, saved_nvalid;   // int32 [B]
-  int64_t commit_path;                   // int32 [B][16]
+  int64_t ctx_len, nvalid, gen_count, commit_base, commit_nv, root;   // int32 [B]
+  int64_t node_ok, node_top;             // int32 [B][128]: the node is among its parent's draws; its own first draw
   int64_t seq_order;                     // int32 [R]: rows by descending context length
   int64_t tree_parent, tree_depth, tree_rank, tree_anc;       // [B*128] (anc: two uint64 per node)
+  int64_t tree_inner;                    // [B*128]: nodes that have children, -1 behind the last
   int64_t chain_parent, chain_depth, chain_rank, chain_anc;   // [128]
   int64_t tokens, stage_tokens;          // int32 [M]
   int64_t kv_row;                        // int64 [M]: element offset of the row's K slot (head 0) in a layer's pool, -1: none
@@ -135,13 +136,12 @@ inline WorkspaceLayout workspace_layout(const vadusa_config* c) {
   auto take = [&](int64_t bytes) { int64_t o = off; off = align_up(off + bytes, 256); return o; };
   w.scalars = take(256);
   w.ctx_len = take(B * 4); w.nvalid = take(B * 4); w.gen_count = take(B * 4);
-  w.commit_base = take(B * 4); w.commit_len = take(B * 4); w.best = take(B * 4); w.root = take(B * 4);
-  w.saved_nvalid = take(B * 4);
-  w.commit_path = take(B * 16 * 4);
+  w.commit_base = take(B * 4); w.commit_nv = take(B * 4); w.root = take(B * 4);
+  w.node_ok = take(B * VADUSA_MAX_TREE_NODES * 4); w.node_top = take(B * VADUSA_MAX_TREE_NODES * 4);
   w.seq_order = take(R * 4);
   const int64_t T = VADUSA_MAX_TREE_NODES;
   w.tree_parent = take(B * T * 4); w.tree_depth = take(B * T * 4); w.tree_rank = take(B * T * 4);
-  w.tree_anc = take(B * T * 16);
+  w.tree_anc = take(B * T * 16); w.tree_inner = take(B * T * 4);
   w.chain_parent = take(T * 4); w.chain_depth = take(T * 4); w.chain_rank = take(T * 4);
   w.chain_anc = take(T * 16);
   w.tokens = take(M * 4); w.stage_tokens = take(M * 4);

@@ -65,7 +65,7 @@ vadusa_status run(unsigned char* scratch, const void* dw, const float* db, const
   sp.eos_masked = eos_masked ? 1 : 0; sp.eos_id = vocab - 1;
   // grid.x = heads only: the select kernel's extra block (the root sample) is not launched
   dim3 g3(heads, batch);
-  draft_select_kernel<<<g3, 256, 0, stream>>>(logits, nullptr, ld, vocab, batch, heads, topk, nullptr, active, sp,
+  draft_select_kernel<<<g3, select_threads(vocab), 0, stream>>>(logits, nullptr, ld, vocab, batch, heads, topk, nullptr, active, sp,
                                               topk_out, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(VADUSA_ECUDA, cudaGetErrorString(e));
