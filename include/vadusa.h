@@ -9,8 +9,8 @@
  *    Any output pointer may be NULL, which means "do not write it".
  *  - The caller owns every buffer it passes (weights, KV pool, workspace, block
  *    table, inputs, outputs) and keeps it alive until vadusa_destroy.  The
- *    library owns only the opaque vadusa_ctx (host memory, two CUDA events and
- *    a few pinned host words).
+ *    library owns only the opaque vadusa_ctx (host memory, a few CUDA events and
+ *    2 MB of pinned host memory for staging).
  *  - All device work is enqueued on the stream given in the configuration, in
  *    call order; calls do not synchronise unless they say so.
  *  - Errors found on the host make the call return at once with a message in
@@ -189,7 +189,9 @@ vadusa_status vadusa_begin(vadusa_ctx *ctx, int32_t batch, const int32_t *block_
  * them, so later chunks of a sequence see the earlier ones of the same pass.
  * h_tokens: host int32 [batch][stride], phoneme p written as vocab + p; h_len: host
  * int32 [batch].  Leaves the hidden state and base-head logits of the last prefix
- * token as the start of decoding.  Synchronises the stream. */
+ * token as the start of decoding.  The host arrays are staged: they may be reused on return, the
+ * work itself is only enqueued (it waits for the device first if commits have moved the context
+ * lengths since vadusa_begin or vadusa_get_lengths). */
 vadusa_status vadusa_prefill(vadusa_ctx *ctx, const int32_t *h_tokens, const int32_t *h_len, int32_t stride);
 
 /* Microbenchmark / test entry: sets the carried state directly.  hstar: [batch][d_model]

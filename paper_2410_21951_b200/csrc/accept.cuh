@@ -24,7 +24,8 @@ struct SeqState {             // device state of the batch (all [batch] unless n
   int32_t* node_ok;           // [batch][kMaxNodes]: the node is among its parent's draws
   int32_t* node_top;          // [batch][kMaxNodes]: the node's first draw, where accept_kernel forms it
   int32_t* out_tokens;        // [batch][out_cap] generated tokens (may be null)
-  int32_t* done_count;        // scalar: sequences that reached the target
+  int32_t* done_count;        // [3] scalars: sequences that reached the target, iterations finished, blocks arrived in this one
+  int32_t* progress;          // pinned host memory [2] that gets (iterations finished, sequences done) after every commit, or null
   int out_cap;
   int target;                 // stop a sequence after this many tokens (0: never)
   unsigned long long* stats;  // [2][kStatDepth][kStatTopk]: acceptance tests applied / passed, by (draft head, rank)
@@ -98,6 +99,18 @@ __global__ void __launch_bounds__(1024) accept_kernel(
   }
 }
 
+// One thread per sequence, after it has counted the sequence's end: the last of the batch tells the host.
+__device__ __forceinline__ void report_progress(const SeqState& st) {
+  if (!st.progress) return;
+  __threadfence();
+  if (atomicAdd(st.done_count + 2, 1) != (int)gridDim.y - 1) return;
+  st.done_count[2] = 0;
+  const int it = st.done_count[1] + 1;
+  st.done_count[1] = it;
+  const unsigned long long both = (uint32_t)it | ((unsigned long long)(uint32_t)atomicAdd(st.done_count, 0) << 32);
+  *reinterpret_cast<volatile unsigned long long*>(st.progress) = both;
+}
+
 // floats of the carried logits that one block of commit_kernel copies
 constexpr int kCommitLogits = 4096;
 
@@ -144,6 +157,7 @@ __global__ void __launch_bounds__(1024) commit_kernel(
       if (out.accept_len) out.accept_len[b] = 0;
       if (out.edge_bits) for (int w = 0; w < (int)out.edge_words; ++w) out.edge_bits[b * out.edge_words + w] = 0ull;
       if (out.next_root) out.next_root[b] = -1;
+      report_progress(st);
     }
     if (tid < kMaxPath) {
       if (out.path_nodes) out.path_nodes[b * kMaxPath + tid] = -1;
@@ -233,6 +247,7 @@ __global__ void __launch_bounds__(1024) commit_kernel(
       if (out.edge_bits)
         for (int w = 0; w < (int)out.edge_words; ++w)
           out.edge_bits[b * out.edge_words + w] = s_acc[2 * w] | ((unsigned long long)s_acc[2 * w + 1] << 32);
+      report_progress(st);
     }
     if (out.next_root && have_top) {
       if (tid == 0) out.next_root[b] = st.node_top[b * kMaxNodes + best];
@@ -283,25 +298,38 @@ __global__ void __launch_bounds__(1024) commit_kernel(
 }
 
 // Prefill bookkeeping.  gather: row r of the pass gets the block-table row of its sequence.
-__global__ void prefill_gather_kernel(const int32_t* __restrict__ block_table, const int32_t* __restrict__ seq_of,
+__global__ void prefill_gather_kernel(const int32_t* __restrict__ block_table, const int32_t* seq_of,
                                       int max_blocks, int32_t* __restrict__ out) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int r = blockIdx.x, b = seq_of[r];
   for (int i = threadIdx.x; i < max_blocks; i += blockDim.x) out[(long long)r * max_blocks + i] = block_table[(long long)b * max_blocks + i];
 }
 
-// finish: the row holding the last chunk of sequence b carries that sequence's state forward: the
-// hidden state and base-head logits of its last token, and the new context length.  grid = rows.
+// pick: rows m[i] of the attention outputs and of the residual stream, one behind the other.  grid = rows.
 template <typename T>
-__global__ void prefill_finish_kernel(const int32_t* __restrict__ row_ctx, const int32_t* __restrict__ row_nvalid,
-                                      const int32_t* __restrict__ row_last, int n_nodes, const T* __restrict__ hfinal,
-                                      int d_model, const float* __restrict__ logits, int ld, T* __restrict__ hstar,
+__global__ void prefill_pick_kernel(const int32_t* m, const T* o, const float* x, int d, T* __restrict__ a, float* __restrict__ xg) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const long long i = blockIdx.x, r = m[i];
+  for (int c = threadIdx.x; c < d * (int)sizeof(T) / 16; c += blockDim.x)
+    reinterpret_cast<uint4*>(a + i * d)[c] = reinterpret_cast<const uint4*>(o + r * d)[c];
+  for (int c = threadIdx.x; c < d / 4; c += blockDim.x)
+    reinterpret_cast<float4*>(xg + i * d)[c] = reinterpret_cast<const float4*>(x + r * d)[c];
+}
+
+// finish: what the last token of a prefix leaves, as its sequence's state: hidden state, base-head logits, context length.
+// by_row: hidden state and logits lie at the token's row of the pass (m), else at the index of the prefix.  grid = ends.
+template <typename T>
+__global__ void prefill_finish_kernel(const int32_t* m, const int32_t* seq, const int32_t* len, int by_row, const T* hfinal,
+                                      int d_model, const float* logits, int ld, T* __restrict__ hstar,
                                       float* __restrict__ logits_star, int32_t* __restrict__ ctx_len) {
-  const int r = blockIdx.x, b = row_last[r], nv = row_nvalid[r];
-  if (b < 0 || nv == 0) return;
-  const long long m = (long long)r * n_nodes + nv - 1;
-  for (int i = threadIdx.x; i < d_model; i += blockDim.x) hstar[(long long)b * d_model + i] = hfinal[m * d_model + i];
-  for (int i = threadIdx.x; i < ld; i += blockDim.x) logits_star[(long long)b * ld + i] = logits[m * ld + i];
-  if (threadIdx.x == 0) ctx_len[b] = row_ctx[r] + nv;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int i = blockIdx.x, b = seq[i];
+  const long long r = by_row ? m[i] : i;
+  for (int c = threadIdx.x; c < d_model * (int)sizeof(T) / 16; c += blockDim.x)
+    reinterpret_cast<uint4*>(hstar + (long long)b * d_model)[c] = reinterpret_cast<const uint4*>(hfinal + r * d_model)[c];
+  for (int c = threadIdx.x; c < ld / 4; c += blockDim.x)
+    reinterpret_cast<float4*>(logits_star + (long long)b * ld)[c] = reinterpret_cast<const float4*>(logits + r * ld)[c];
+  if (threadIdx.x == 0) ctx_len[b] = len[i];
 }
 
 }  // namespace vadusa

@@ -48,6 +48,7 @@ struct vadusa_ctx {
   int logit_bias_ld = 0;
   int n_nodes = 0;            // current tree size (0: none set)
   int tree_per_seq = 0;
+  int tree_copies = 1;        // trees in the workspace's tree area (packed: see vadusa_set_tree)
   int max_rank_used = 0;
   int tree_max_depth = 0;
   int tree_inner = 0;         // most nodes with children of any of the trees
@@ -57,7 +58,8 @@ struct vadusa_ctx {
   float fit_lambda = 0.f, fit_lr = 0.f;
   void* pf_tap = nullptr;     // where prefill also leaves the final hidden state of every prefix token ([batch][stride][d])
   int pf_tap_stride = 0;
-  int pf_tiles = 0;           // > 0 while a prefill pass runs: attention CTAs of the pass (pairs of chunks), listed in ws.pf_pairs
+  int pf_tiles = 0;           // > 0 while a prefill pass runs: attention CTAs of the pass (pairs of chunks), listed in pf_pairs
+  const int2* pf_pairs = nullptr;
   int att_stream = 0;         // batches: attention as one persistent kernel over the stream of K/V pages (0: one CTA per head and sequence)
   int fused_enabled = 0;      // single-sequence passes run as one persistent kernel (0: no, 1: yes, 6 / 8: with that cluster size)
   int fused_clusters = -1;    // clusters of that kernel that can be resident at once on this device (-1: not asked yet)
@@ -68,15 +70,27 @@ struct vadusa_ctx {
   const int32_t* block_table = nullptr;
   bool have_draft = false, have_verify = false;
   int64_t launches = 0;
-  cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_poll = nullptr;
-  int32_t* h_pinned = nullptr;     // [2]: done_count, err
+  cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  // Host-visible words: the generation loop's progress (see run_generate), then the sequences' token counts and error word
+  int32_t* h_pinned = nullptr;
+  // Pinned staging of host arrays on their way to the device: two halves, each with an event behind its last copy, so
+  // that a call returns as soon as its arrays are staged instead of waiting for the stream
+  char* up = nullptr;
+  size_t up_at = 0;
+  int up_half = 0;
+  bool up_used[2] = {false, false};
+  cudaEvent_t ev_up[2] = {nullptr, nullptr};
+  // context lengths as the host knows them (exact after begin, prefill, get_lengths and generate)
+  std::vector<int32_t> h_ctx;
+  bool h_ctx_exact = false;
   char err[512] = {0};
   // TMA descriptors of the operands of the tensor-core products, made on first use
   typedef std::tuple<const void*, int, int, int, int, long long> MapKey;   // ptr, rows, K, box rows, batches, batch stride
   std::map<MapKey, CUtensorMap> maps;
   void* encode_fn = nullptr;       // cuTensorMapEncodeTiled, resolved through the runtime
   // CUDA graphs of the launch sequences of the hot calls, keyed by their baked-in arguments
-  struct GraphRec { cudaGraphExec_t exec = nullptr; int seen = 0; int64_t launches = 0; };
+  struct GraphRec { cudaGraphExec_t exec = nullptr; int seen = 0; int64_t launches = 0, used = 0; };
+  int64_t graph_clock = 0;
   std::map<std::string, GraphRec> graphs;
   // per-kernel timing (vadusa_profile_begin/end): one event pair per launch
   struct ProfRec { cudaEvent_t a, b; int cls; };
@@ -182,10 +196,12 @@ TreeView tree_of(vadusa_ctx* c, bool chain) {
     t.n_nodes = c->cfg.max_tree_nodes;
     t.per_seq = 0;
   } else {
-    t.parent = wsptr<int32_t>(c, c->ws.tree_parent);
-    t.depth = wsptr<int32_t>(c, c->ws.tree_depth);
-    t.rank = wsptr<int32_t>(c, c->ws.tree_rank);
-    t.anc = wsptr<unsigned long long>(c, c->ws.tree_anc);
+    const size_t nn = (size_t)c->tree_copies * c->n_nodes;
+    t.parent = wsptr<int32_t>(c, c->ws.tree);
+    t.depth = t.parent + nn;
+    t.rank = t.depth + nn;
+    t.anc = reinterpret_cast<const unsigned long long*>(
+        c->wsp + c->ws.tree + ((nn * 12 + (size_t)c->tree_copies * VADUSA_MAX_TREE_NODES * 4 + 15) & ~(size_t)15));
     t.n_nodes = c->n_nodes;
     t.per_seq = c->tree_per_seq;
   }
@@ -230,6 +246,30 @@ vadusa_status sampling_dev(vadusa_ctx* ctx, const vadusa_sampling* s, SamplingDe
   return VADUSA_OK;
 }
 
+constexpr size_t kUpHalf = 1 << 20;
+constexpr int kHostWords = 4;       // h_pinned: iterations finished, sequences done, error word, unused; then [batch] token counts
+
+// Copies `bytes` from host memory (the caller's, free again on return) to dst in stream order.
+vadusa_status upload(vadusa_ctx* ctx, void* dst, const void* src, size_t bytes) {
+  if (bytes > kUpHalf) {
+    CU(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    return VADUSA_OK;
+  }
+  if (ctx->up_at + bytes > kUpHalf) {
+    CU(cudaEventRecord(ctx->ev_up[ctx->up_half], ctx->stream));
+    ctx->up_used[ctx->up_half] = true;
+    ctx->up_half ^= 1;
+    ctx->up_at = 0;
+    if (ctx->up_used[ctx->up_half]) CU(cudaEventSynchronize(ctx->ev_up[ctx->up_half]));
+  }
+  char* at = ctx->up + ctx->up_half * kUpHalf + ctx->up_at;
+  memcpy(at, src, bytes);
+  ctx->up_at += (bytes + 15) & ~(size_t)15;
+  CU(cudaMemcpyAsync(dst, at, bytes, cudaMemcpyHostToDevice, ctx->stream));
+  return VADUSA_OK;
+}
+
 // Launch of a kernel that begins with griddepcontrol.wait: it may be set up while its predecessor is still running.
 template <typename K, typename... A>
 cudaError_t launch_dependent(vadusa_ctx* ctx, K kernel, dim3 grid, int threads, size_t smem, A... args) {
@@ -247,12 +287,20 @@ cudaError_t launch_dependent(vadusa_ctx* ctx, K kernel, dim3 grid, int threads, 
 
 // ---- typed engine ------------------------------------------------------------------
 
+// Plain FMA product; rn: LayerNorm of the operand rows on the way (few tokens only).
 template <typename T, typename Epi>
 vadusa_status gemm(vadusa_ctx* ctx, int cls, const T* A, const T* W, int M, int N, int K, int batches, long long a_z,
-                   long long w_z, const Epi& epi) {
-  dim3 grid((N + 63) / 64, (M + 63) / 64, batches);
+                   long long w_z, const Epi& epi, const RowNorm* rn = nullptr) {
   PROF(ctx, cls);
-  gemm_simt_kernel<T, Epi><<<grid, 256, 0, ctx->stream>>>(A, W, M, N, K, a_z, w_z, epi);
+  if (M <= kFewTokens) {
+    const int mw = M <= 4 ? 1 : M <= 8 ? 2 : 4, nw = 4 / mw;         // warps of a block along tokens / features
+    const dim3 grid((N + 4 * nw - 1) / (4 * nw), (M + 4 * mw - 1) / (4 * mw), batches);
+    if (rn) CU(launch_dependent(ctx, gemm_few_kernel<T, Epi, true>, grid, 128, 0, A, W, M, N, K, a_z, w_z, mw, epi, *rn));
+    else CU(launch_dependent(ctx, gemm_few_kernel<T, Epi, false>, grid, 128, 0, A, W, M, N, K, a_z, w_z, mw, epi, RowNorm{}));
+  } else {
+    CU(launch_dependent(ctx, gemm_simt_kernel<T, Epi>, dim3((N + 63) / 64, (M + 63) / 64, batches), 256, 0, A, W, M, N, K, a_z,
+                        w_z, epi));
+  }
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
@@ -473,11 +521,18 @@ vadusa_status product(vadusa_ctx* ctx, int cls, const T* X, const T* W, int w_ro
   return gemm<T>(ctx, cls, X, W, M, N, K, batches, x_z, w_z, epi);
 }
 
-// LayerNorm followed by a product, in one kernel where the shape allows (bf16 models, few tokens).
+// LayerNorm followed by a product, in one kernel where the shape allows (few tokens; bf16: from the statistics that the
+// producer of x left).
 template <typename T, typename Epi>
 bool ln_product(vadusa_ctx* ctx, int cls, const float* x, const float* g, const float* b, const T* W, int w_rows, int M,
                 int N, int K, const Epi& epi, vadusa_status* st, T* y = nullptr) {
   if constexpr (std::is_same<T, bf16>::value) return gemm_tc_ln(ctx, cls, x, g, b, W, w_rows, M, N, K, epi, st, y);
+  if constexpr (std::is_same<T, float>::value) {
+    if (M > kFewTokens || K > kFewNormK) return false;
+    const RowNorm rn{g, b, y, ctx->cfg.ln_eps};
+    *st = gemm<float>(ctx, cls, x, W, M, N, K, 1, 0, 0, epi, &rn);
+    return true;
+  }
   return false;
 }
 
@@ -510,13 +565,13 @@ vadusa_status attention(vadusa_ctx* ctx, const T* q, const T* pool, const TreeVi
   const KvGeom g = geom_of(ctx);
   const float scale = (float)(1.0 / sqrt((double)dh));
   const int ntile = (tv.n_nodes + 63) / 64;
-  dim3 grid(c.n_heads, ctx->batch * ntile);
-  const size_t smem = (size_t)(64 * dh * 3 + 64 + 64 * 64) * sizeof(float);   // = attention_smem(dh)
+  // four nodes per block while that makes at most four blocks per SM, else eight
+  const int ng = c.n_heads * ctx->batch * ((tv.n_nodes + 3) / 4) <= 4 * 148 ? 4 : 8;
   auto go = [&](auto kern) -> vadusa_status {
     PROF(ctx, K_ATTENTION);
-    kern<<<grid, 256, smem, ctx->stream>>>(q, pool, ctx->block_table, wsptr<int32_t>(ctx, ctx->ws.ctx_len),
-                                           wsptr<int32_t>(ctx, ctx->ws.nvalid), tv, g, c.d_model, scale, out,
-                                           err_word(ctx));
+    CU(launch_dependent(ctx, kern, dim3(c.n_heads, ctx->batch, (tv.n_nodes + ng - 1) / ng), 256, att_simt_smem(dh), q, pool, ctx->block_table,
+                        (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.ctx_len), (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.nvalid),
+                        tv, g, c.d_model, scale, out, err_word(ctx)));
     LAUNCH_CHECK();
     return VADUSA_OK;
   };
@@ -545,7 +600,7 @@ vadusa_status attention(vadusa_ctx* ctx, const T* q, const T* pool, const TreeVi
         CU(cudaLaunchKernelEx(&lc, prefill_attention_tc_kernel, *mq, *mkv, layer, ctx->block_table,
                               (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.ctx_len),
                               (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.nvalid),
-                              (const int2*)wsptr<int2>(ctx, ctx->ws.pf_pairs), g, c.d_model,
+                              ctx->pf_pairs, g, c.d_model,
                               scale * 1.4426950408889634f, reinterpret_cast<bf16*>(out), err_word(ctx)));
         LAUNCH_CHECK();
         return VADUSA_OK;
@@ -602,8 +657,10 @@ vadusa_status attention(vadusa_ctx* ctx, const T* q, const T* pool, const TreeVi
       return VADUSA_OK;
     }
   }
-  if (dh == 64) return go(tree_attention_simt_kernel<T, 64>);
-  return go(tree_attention_simt_kernel<T, 32>);
+  if constexpr (!std::is_same<T, bf16>::value) {
+    if (dh == 64) return ng == 4 ? go(tree_attention_simt_kernel<T, 64, 4>) : go(tree_attention_simt_kernel<T, 64, 8>);
+  }
+  return ng == 4 ? go(tree_attention_simt_kernel<T, 32, 4>) : go(tree_attention_simt_kernel<T, 32, 8>);
 }
 
 template <typename T>
@@ -752,9 +809,46 @@ vadusa_status embed(vadusa_ctx* ctx, const TreeView& tv, const int32_t* override
   return VADUSA_OK;
 }
 
-// One forward pass of the base model over batch * tv.n_nodes rows (verify step).
+// The rows of a prefill pass that the last layer is needed for: the last token of every prefix that ends in the pass.
+struct PrefillTail {
+  int rows;                  // 0: no prefix ends here
+  int tiles;                 // attention tiles that hold these rows
+  const int2* pairs;
+  const int32_t* m;          // device [rows]: row of the pass
+};
+
+// Everything behind the last layer's q/k/v product for those rows alone: the other rows of that layer only leave K/V behind.
+// (One layer of twelve and the vocabulary head for a few rows: a tenth of a long prefill's work.)
 template <typename T>
-vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* override_tokens, T* attn_tap) {
+vadusa_status prefill_tail(vadusa_ctx* ctx, const TreeView& tv, const PrefillTail& t, const T* pool) {
+  const vadusa_config& c = ctx->cfg;
+  const int d = c.d_model, f = c.d_ffn, vp = vpad(&c), n = t.rows;
+  if (n == 0) return VADUSA_OK;
+  const LayerW& w = ctx->layers[c.n_layers - 1];
+  float* xg = wsptr<float>(ctx, ctx->ws.q);               // (q is free once attention has run)
+  T *a = wsptr<T>(ctx, ctx->ws.a), *o = wsptr<T>(ctx, ctx->ws.o), *mid = wsptr<T>(ctx, ctx->ws.mid), *hf = wsptr<T>(ctx, ctx->ws.hfinal);
+  if (ctx->pf_tiles > 0) { ctx->pf_tiles = t.tiles; ctx->pf_pairs = t.pairs; }
+  if (vadusa_status s = attention<T>(ctx, wsptr<T>(ctx, ctx->ws.q), pool, tv, o)) return s;
+  CU(launch_dependent(ctx, prefill_pick_kernel<T>, dim3(n), 128, 0, t.m, (const T*)o, (const float*)wsptr<float>(ctx, ctx->ws.x), d, a, xg));
+  LAUNCH_CHECK();
+  vadusa_status s = product<T>(ctx, K_GEMM_OUT, a, as<T>(w.wo), d, n, d, d, 1, 0, 0, EpiResidual{w.bo, xg, d});
+  if (s) return s;
+  const EpiRelu<T> e1{w.b1, mid, f};
+  bool fused = std::is_same<T, float>::value && ln_product<T>(ctx, K_GEMM_FFN1, xg, w.ln2_g, w.ln2_b, as<T>(w.w1), f, n, f, d, e1, &s);
+  if (!fused) {
+    if ((s = layernorm<T>(ctx, xg, w.ln2_g, w.ln2_b, o, n))) return s;
+    s = product<T>(ctx, K_GEMM_FFN1, o, as<T>(w.w1), f, n, f, d, 1, 0, 0, e1);
+  }
+  if (s) return s;
+  if ((s = product<T>(ctx, K_GEMM_FFN2, mid, as<T>(w.w2), d, n, d, f, 1, 0, 0, EpiResidual{w.b2, xg, d}))) return s;
+  if ((s = layernorm<T>(ctx, xg, ctx->lnf_g, ctx->lnf_b, hf, n))) return s;
+  return product<T>(ctx, K_GEMM_LM, hf, as<T>(ctx->lm), vp, n, vp, d, 1, 0, 0, EpiLogits{wsptr<float>(ctx, ctx->ws.logits), vp, 0});
+}
+
+// One forward pass of the base model over batch * tv.n_nodes rows (verify step; with `tail` a prefill pass).
+template <typename T>
+vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* override_tokens, T* attn_tap,
+                      const PrefillTail* tail = nullptr) {
   const vadusa_config& c = ctx->cfg;
   const int B = ctx->batch, N = tv.n_nodes, M = B * N, d = c.d_model, f = c.d_ffn, vp = vpad(&c);
   const KvGeom g = geom_of(ctx);
@@ -780,7 +874,7 @@ vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* overri
   const bool stats_out = tc && residual_leaves_stats(M, d, d), stats_ffn = tc && residual_leaves_stats(M, d, f);
   float2* stats = wsptr<float2>(ctx, ctx->ws.ln_stats);
   if (vadusa_status s = embed<T>(ctx, tv, override_tokens, wsptr<long long>(ctx, ctx->ws.kv_row), embed_stats ? stats : nullptr)) return s;
-  bool have_stats = embed_stats;
+  bool have_stats = embed_stats || !tc;                    // (fp32 models need none)
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerW& w = ctx->layers[l];
     T* pool = reinterpret_cast<T*>(c.kv_pool) + (long long)l * g.layer_stride;
@@ -793,6 +887,7 @@ vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* overri
       s = product<T>(ctx, K_GEMM_QKV, a, as<T>(w.wqkv), 3 * d, M, 3 * d, d, 1, 0, 0, eq);
     }
     if (s) return s;
+    if (tail && l == c.n_layers - 1) return prefill_tail<T>(ctx, tv, *tail, pool);
     s = attention<T>(ctx, q, pool, tv, o);
     if (s) return s;
     if (attn_tap)
@@ -820,7 +915,7 @@ vadusa_status forward(vadusa_ctx* ctx, const TreeView& tv, const int32_t* overri
       EpiResidual e2{w.b2, x, d};
       s = product<T>(ctx, K_GEMM_FFN2, mid, as<T>(w.w2), d, M, d, f, 1, 0, 0, e2);
     }
-    have_stats = stats_ffn;
+    have_stats = stats_ffn || !tc;
     if (s) return s;
   }
   EpiLogits el{logits, vp, 0};
@@ -861,12 +956,13 @@ vadusa_status draft(vadusa_ctx* ctx, const SamplingDev& sp) {
 // tokens = tree built from the draft (no model pass): used when the caller wants them.
 template <typename T>
 vadusa_status accept_commit(vadusa_ctx* ctx, const SamplingDev& sp, const int32_t* forced, const AcceptOut& out,
-                            int32_t* out_tokens, int out_cap, int target) {
+                            int32_t* out_tokens, int out_cap, int target, int32_t* progress = nullptr) {
   const vadusa_config& c = ctx->cfg;
   const int B = ctx->batch, vp = vpad(&c);
   const KvGeom g = geom_of(ctx);
   const TreeView tv = tree_of(ctx, false);
   SeqState st = state_of(ctx, out_tokens, out_cap, target);
+  st.progress = progress;
   PROF(ctx, K_ACCEPT);
   // the next root is wanted and the device holds a block per node at once: every node's first draw along with the rest
   const bool tops = out.next_root && sp.accept_rule == 0 && tv.n_nodes * B <= 2 * 148;
@@ -874,7 +970,7 @@ vadusa_status accept_commit(vadusa_ctx* ctx, const SamplingDev& sp, const int32_
   CU(launch_dependent(ctx, accept_kernel, dim3(tops ? tv.n_nodes : ctx->tree_inner, B), accept_threads(c.vocab, tv.n_nodes * B), row_keys_smem(vp, sp),
                       (const float*)wsptr<float>(ctx, ctx->ws.logits), vp, c.vocab,
                       (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.tokens), tv,
-                      (const int32_t*)(tops ? nullptr : wsptr<int32_t>(ctx, ctx->ws.tree_inner)), sp, st));
+                      (const int32_t*)(tops ? nullptr : wsptr<int32_t>(ctx, ctx->ws.tree) + 3ll * ctx->tree_copies * tv.n_nodes), sp, st));
   LAUNCH_CHECK();
   PROF(ctx, K_COMMIT);
   CU(launch_dependent(ctx, commit_kernel<T>, dim3(c.n_layers + (vp + kCommitLogits - 1) / kCommitLogits + 1, B),
@@ -897,6 +993,22 @@ struct RowsView {
   ~RowsView() { c->batch = batch; c->block_table = table; c->ws.ctx_len = ctx_len; c->ws.nvalid = nvalid; }
 };
 
+// A prefill pass's arrays in ws.pf_stage, packed behind one another so that one copy brings them.
+struct PassArrays {
+  int rows, n_nodes;
+  size_t pairs() const { return 0; }                            // int2: rows that share an attention CTA (y < 0: a single chunk)
+  size_t tail_pairs() const { return (size_t)rows * 8; }        // int2: those of them that hold the end of a prefix
+  size_t word(int i) const { return (size_t)rows * (16 + 4 * i); }
+  size_t ctx() const { return word(0); }                        // int32: tokens before the chunk
+  size_t nvalid() const { return word(1); }                     // its length
+  size_t seq() const { return word(2); }                        // its sequence
+  size_t tail_m() const { return word(3); }                     // [tail]: row of a prefix's last token,
+  size_t tail_seq() const { return word(4); }                   //         its sequence,
+  size_t tail_len() const { return word(5); }                   //         and the sequence's new length
+  size_t tokens() const { return word(6); }                     // int32 [rows][n_nodes]
+  size_t total() const { return tokens() + (size_t)rows * n_nodes * 4; }
+};
+
 template <typename T>
 vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h_len, int stride) {
   const vadusa_config& c = ctx->cfg;
@@ -904,12 +1016,16 @@ vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h
   int longest = 0;
   for (int b = 0; b < B; ++b) {
     if (h_len[b] < 1 || h_len[b] > stride) return fail(ctx, VADUSA_EINVAL, "prefix length of sequence %d out of range", b);
+    if (ctx->pf_tap && h_len[b] > ctx->pf_tap_stride) return fail(ctx, VADUSA_EINVAL, "prefill tap: row stride shorter than the prefix");
     longest = h_len[b] > longest ? h_len[b] : longest;
   }
   // what the cache holds already
-  std::vector<int32_t> base(B);
-  CU(cudaMemcpyAsync(base.data(), ctx->wsp + ctx->ws.ctx_len, B * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
+  if (!ctx->h_ctx_exact) {
+    ctx->h_ctx.resize(B);
+    CU(cudaMemcpyAsync(ctx->h_ctx.data(), ctx->wsp + ctx->ws.ctx_len, B * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    ctx->h_ctx_exact = true;
+  }
   // chunks in sequence order, so that a chunk never precedes an earlier chunk of its sequence
   struct Chunk { int b, s0, n, last; };
   std::vector<Chunk> chunks;
@@ -918,65 +1034,74 @@ vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h
       const int n = h_len[b] - s0 < N ? h_len[b] - s0 : N;
       chunks.push_back({b, s0, n, s0 + n == h_len[b] ? b : -1});
     }
-  int32_t* d_stage = wsptr<int32_t>(ctx, ctx->ws.stage_tokens);
-  int32_t* d_ctx = wsptr<int32_t>(ctx, ctx->ws.pf_ctx_len);
-  int32_t* d_nv = wsptr<int32_t>(ctx, ctx->ws.pf_nvalid);
-  int32_t* d_seq = wsptr<int32_t>(ctx, ctx->ws.pf_seq);
-  int32_t* d_last = wsptr<int32_t>(ctx, ctx->ws.pf_last);
   int32_t* d_table = wsptr<int32_t>(ctx, ctx->ws.pf_block_table);
   int32_t* real_ctx_len = wsptr<int32_t>(ctx, ctx->ws.ctx_len);
   const int32_t* real_table = ctx->block_table;
-  std::vector<int32_t> stage((size_t)R * N), v_ctx(R), v_nv(R), v_seq(R), v_last(R), v_pairs(2 * (size_t)R);
+  std::vector<char> pack;
   const TreeView tv = tree_of(ctx, true);
   for (size_t c0 = 0; c0 < chunks.size(); c0 += R) {
     const int rows = (int)(chunks.size() - c0 < (size_t)R ? chunks.size() - c0 : R);
+    const PassArrays pa{rows, N};
+    pack.assign(pa.total(), 0);
+    auto at = [&](size_t off) { return reinterpret_cast<int32_t*>(pack.data() + off); };
+    int ends = 0;
     for (int r = 0; r < rows; ++r) {
       const Chunk& ch = chunks[c0 + r];
-      v_ctx[r] = base[ch.b] + ch.s0; v_nv[r] = ch.n; v_seq[r] = ch.b; v_last[r] = ch.last;
-      for (int i = 0; i < N; ++i) stage[(size_t)r * N + i] = i < ch.n ? h_tokens[(size_t)ch.b * stride + ch.s0 + i] : 0;
+      at(pa.ctx())[r] = ctx->h_ctx[ch.b] + ch.s0; at(pa.nvalid())[r] = ch.n; at(pa.seq())[r] = ch.b;
+      if (ch.last >= 0) {
+        at(pa.tail_m())[ends] = r * N + ch.n - 1; at(pa.tail_seq())[ends] = ch.b;
+        at(pa.tail_len())[ends] = ctx->h_ctx[ch.b] + ch.s0 + ch.n;
+        ++ends;
+      }
+      memcpy(at(pa.tokens()) + (size_t)r * N, h_tokens + (size_t)ch.b * stride + ch.s0, ch.n * sizeof(int32_t));
     }
-    CU(cudaMemcpyAsync(d_ctx, v_ctx.data(), rows * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(d_nv, v_nv.data(), rows * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(d_seq, v_seq.data(), rows * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(d_last, v_last.data(), rows * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(d_stage, stage.data(), (size_t)rows * N * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
     // attention tiles of the pass: a full chunk and the chunk behind it in the same sequence share a CTA
-    int tiles = 0;
+    int tiles = 0, tail_tiles = 0;
     for (int r = 0; r < rows;) {
       const Chunk& ch = chunks[c0 + r];
       const bool pair = r + 1 < rows && chunks[c0 + r + 1].b == ch.b && ch.n == N;
-      v_pairs[2 * tiles] = r; v_pairs[2 * tiles + 1] = pair ? r + 1 : -1;
+      at(pa.pairs())[2 * tiles] = r; at(pa.pairs())[2 * tiles + 1] = pair ? r + 1 : -1;
       ++tiles;
+      if (ch.last >= 0 || (pair && chunks[c0 + r + 1].last >= 0)) {
+        at(pa.tail_pairs())[2 * tail_tiles] = r; at(pa.tail_pairs())[2 * tail_tiles + 1] = pair ? r + 1 : -1;
+        ++tail_tiles;
+      }
       r += pair ? 2 : 1;
     }
-    CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.pf_pairs, v_pairs.data(), (size_t)tiles * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));   // the staging vectors are reused by the next pass
-    prefill_gather_kernel<<<rows, 128, 0, ctx->stream>>>(real_table, d_seq, c.max_blocks_per_seq, d_table);
+    char* dev = ctx->wsp + ctx->ws.pf_stage;
+    if (vadusa_status s = upload(ctx, dev, pack.data(), pack.size())) return s;
+    auto dp = [&](size_t off) { return reinterpret_cast<int32_t*>(dev + off); };
+    CU(launch_dependent(ctx, prefill_gather_kernel, dim3(rows), 128, 0, real_table, (const int32_t*)dp(pa.seq()), c.max_blocks_per_seq, d_table));
     LAUNCH_CHECK();
+    // (the persistent pass has no tail of its own; the gathered residual rows take the place of q)
+    const bool whole = ctx->pf_tap != nullptr || ctx->fused_enabled || (size_t)ends * 4 > (size_t)rows * N * sizeof(T);
     {
-      RowsView view(ctx, rows, d_table, ctx->ws.pf_ctx_len, ctx->ws.pf_nvalid);
+      RowsView view(ctx, rows, d_table, ctx->ws.pf_stage + (int64_t)pa.ctx(), ctx->ws.pf_stage + (int64_t)pa.nvalid());
+      const PrefillTail tail{ends, tail_tiles, reinterpret_cast<const int2*>(dev + pa.tail_pairs()), dp(pa.tail_m())};
       ctx->pf_tiles = tiles;
-      const vadusa_status s = forward<T>(ctx, tv, d_stage, nullptr);
+      ctx->pf_pairs = reinterpret_cast<const int2*>(dev + pa.pairs());
+      const vadusa_status s = forward<T>(ctx, tv, dp(pa.tokens()), nullptr, whole ? nullptr : &tail);
       ctx->pf_tiles = 0;
       if (s) return s;
     }
-    prefill_finish_kernel<T><<<rows, 256, 0, ctx->stream>>>(d_ctx, d_nv, d_last, N, wsptr<T>(ctx, ctx->ws.hfinal), c.d_model,
-                                                            wsptr<float>(ctx, ctx->ws.logits), vp,
-                                                            wsptr<T>(ctx, ctx->ws.hstar),
-                                                            wsptr<float>(ctx, ctx->ws.logits_star), real_ctx_len);
-    LAUNCH_CHECK();
+    if (ends > 0) {
+      CU(launch_dependent(ctx, prefill_finish_kernel<T>, dim3(ends), 256, 0, (const int32_t*)dp(pa.tail_m()), (const int32_t*)dp(pa.tail_seq()),
+                          (const int32_t*)dp(pa.tail_len()), whole ? 1 : 0, (const T*)wsptr<T>(ctx, ctx->ws.hfinal), c.d_model,
+                          (const float*)wsptr<float>(ctx, ctx->ws.logits), vp, wsptr<T>(ctx, ctx->ws.hstar),
+                          wsptr<float>(ctx, ctx->ws.logits_star), real_ctx_len));
+      LAUNCH_CHECK();
+    }
     if (ctx->pf_tap)
       for (int r = 0; r < rows; ++r) {
         const Chunk& ch = chunks[c0 + r];
-        if (ch.s0 + ch.n > ctx->pf_tap_stride) return fail(ctx, VADUSA_EINVAL, "prefill tap: row stride shorter than the prefix");
         CU(cudaMemcpyAsync(reinterpret_cast<T*>(ctx->pf_tap) + ((long long)ch.b * ctx->pf_tap_stride + ch.s0) * c.d_model,
                            wsptr<T>(ctx, ctx->ws.hfinal) + (long long)r * N * c.d_model, (size_t)ch.n * c.d_model * sizeof(T),
                            cudaMemcpyDeviceToDevice, ctx->stream));
       }
   }
+  for (int b = 0; b < B; ++b) ctx->h_ctx[b] += h_len[b];
   ctx->ctx_bound += longest;
   ctx->ctx_lo += longest;
-  CU(cudaStreamSynchronize(ctx->stream));
   return VADUSA_OK;
 }
 
@@ -1072,13 +1197,14 @@ vadusa_status fit_step(vadusa_ctx* ctx, const FitLayout& f, const T* hidden, con
   return VADUSA_OK;
 }
 
-size_t attention_smem(int dh) { return (size_t)(64 * dh * 3 + 64 + 64 * 64) * sizeof(float); }
-
 vadusa_status set_kernel_attributes(vadusa_ctx* ctx) {
-  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<float, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_smem(64)));
-  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<float, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_smem(32)));
-  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<bf16, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_smem(64)));
-  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<bf16, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attention_smem(32)));
+  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<float, 64, 4>, smem, att_simt_smem(64)));
+  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<float, 64, 8>, smem, att_simt_smem(64)));
+  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<float, 32, 4>, smem, att_simt_smem(32)));
+  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<float, 32, 8>, smem, att_simt_smem(32)));
+  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<bf16, 32, 4>, smem, att_simt_smem(32)));
+  CU(cudaFuncSetAttribute(tree_attention_simt_kernel<bf16, 32, 8>, smem, att_simt_smem(32)));
   CU(cudaFuncSetAttribute(tree_attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemBytes));
   CU(cudaFuncSetAttribute(prefill_attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemBytes));
   CU(cudaFuncSetAttribute(tree_attention_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAsSmemBytes));
@@ -1096,6 +1222,22 @@ vadusa_status set_kernel_attributes(vadusa_ctx* ctx) {
   return VADUSA_OK;
 }
 
+__global__ void begin_kernel(uint32_t* scalars /*[64]*/, uint32_t* f_sync /*[64]*/, uint32_t* att_cnt, int n_cnt, int32_t* gen_count,
+                             int32_t* ctx_len /*or null*/, int32_t* nvalid, int batch, int n_nodes) {
+  const int t = threadIdx.x;
+  if (t < 64) { scalars[t] = 0u; f_sync[t] = 0u; }
+  for (int i = t; i < n_cnt; i += blockDim.x) att_cnt[i] = 0u;
+  for (int b = t; b < batch; b += blockDim.x) {
+    gen_count[b] = 0; nvalid[b] = n_nodes;
+    if (ctx_len) ctx_len[b] = 0;
+  }
+}
+
+__global__ void generate_begin_kernel(int32_t* gen_count, int32_t* nvalid, int batch, int n_nodes, int32_t* done /*[3]: done, iterations, arrived*/) {
+  if (threadIdx.x < 3) done[threadIdx.x] = 0;
+  for (int b = threadIdx.x; b < batch; b += blockDim.x) { gen_count[b] = 0; nvalid[b] = n_nodes; }
+}
+
 __global__ void fill_i32_kernel(int32_t* p, int n, int32_t v) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
@@ -1108,14 +1250,18 @@ vadusa_status set_active(vadusa_ctx* ctx, int value) {
   return VADUSA_OK;
 }
 
-vadusa_status device_errors(vadusa_ctx* ctx) {
-  uint32_t e = 0;
-  CU(cudaMemcpyAsync(&e, err_word(ctx), sizeof(e), cudaMemcpyDeviceToHost, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
+vadusa_status error_of(vadusa_ctx* ctx, uint32_t e) {
   if (e & kErrTimeout) return fail(ctx, VADUSA_ETIMEOUT, "a bounded device-side wait expired (error word 0x%x)", e);
   if (e & kErrCapacity)
     return fail(ctx, VADUSA_ECAPACITY, "a sequence ran past its KV blocks, the position table or the token range (error word 0x%x)", e);
   return VADUSA_OK;
+}
+
+vadusa_status device_errors(vadusa_ctx* ctx) {
+  uint32_t e = 0;
+  CU(cudaMemcpyAsync(&e, err_word(ctx), sizeof(e), cudaMemcpyDeviceToHost, ctx->stream));
+  CU(cudaStreamSynchronize(ctx->stream));
+  return error_of(ctx, e);
 }
 
 // Key of a launch sequence: a tag plus the raw bytes of everything baked into its kernels' arguments.
@@ -1131,11 +1277,16 @@ struct KeyBuilder {
 template <typename F>
 vadusa_status run_graphed(vadusa_ctx* ctx, const std::string& key, F&& body) {
   if (ctx->stream == nullptr || ctx->prof_on) return body();
-  if (ctx->graphs.size() > 64) {
-    for (auto& kv : ctx->graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
-    ctx->graphs.clear();
+  if (ctx->graphs.size() > 64 && ctx->graphs.find(key) == ctx->graphs.end()) {
+    // the sequence that was asked for longest ago makes room
+    auto old = ctx->graphs.begin();
+    for (auto it = ctx->graphs.begin(); it != ctx->graphs.end(); ++it)
+      if (it->second.used < old->second.used) old = it;
+    if (old->second.exec) cudaGraphExecDestroy(old->second.exec);
+    ctx->graphs.erase(old);
   }
   vadusa_ctx::GraphRec& r = ctx->graphs[key];
+  r.used = ++ctx->graph_clock;
   if (r.exec) {
     CU(cudaGraphLaunch(r.exec, ctx->stream));
     ctx->launches += r.launches;
@@ -1169,6 +1320,94 @@ vadusa_status need_batch(vadusa_ctx* ctx) {
   if (!ctx) return VADUSA_EINVAL;
   if (ctx->batch == 0) return fail(ctx, VADUSA_ESTATE, "vadusa_begin has not been called");
   return VADUSA_OK;
+}
+
+// The words in h_pinned, written by the device while the host looks on.
+struct HostWords { volatile int32_t iters, done; volatile uint32_t err; int32_t unused; volatile int32_t gen[1]; };
+
+// out_len[b] = min(gen_count[b], cap); token counts and the error word to the host.  One block.
+__global__ void generate_end_kernel(const int32_t* gen_count, const uint32_t* err, int batch, int cap, int32_t* out_len /*or null*/,
+                                    HostWords* host) {
+  for (int b = threadIdx.x; b < batch; b += blockDim.x) {
+    const int g = gen_count[b];
+    host->gen[b] = g;
+    if (out_len) out_len[b] = g < cap ? g : cap;
+  }
+  if (threadIdx.x == 0) host->err = *err;
+}
+
+// The decoding loop.  The host stays one iteration ahead of the device: the commit of an iteration leaves (iterations
+// finished, sequences done) in pinned host memory, and iteration k is enqueued once k - 2 has been reported, so that the
+// device always has one queued and the loop ends with at most one iteration that finds nothing to do (with a copy and an
+// event every eighth iteration up to sixteen ran behind the end: a quarter of a short request).
+// h_out_tokens / h_out_len: host destinations, or null (then out_len, a device pointer, or null).
+vadusa_status run_generate(vadusa_ctx* ctx, const vadusa_sampling* sampling, int32_t max_new_tokens, int32_t max_iters,
+                           int32_t* out_tokens, int32_t* out_len, int32_t* h_out_tokens, int32_t* h_out_len, vadusa_stats* h_stats) {
+  if (vadusa_status s = need_batch(ctx)) return s;
+  if (ctx->n_nodes == 0 || ctx->tree_per_seq) return fail(ctx, VADUSA_ESTATE, "generate needs a shared tree template");
+  if (max_new_tokens < 1) return fail(ctx, VADUSA_EINVAL, "max_new_tokens must be positive");
+  SamplingDev sp;
+  if (vadusa_status s = sampling_dev(ctx, sampling, &sp)) return s;
+  const int64_t launches0 = ctx->launches;
+  const int limit = max_iters > 0 ? max_iters : max_new_tokens;
+  const TreeView tv = tree_of(ctx, false);
+  AcceptOut none{nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr};
+  HostWords* host = reinterpret_cast<HostWords*>(ctx->h_pinned);
+  // (nothing of an earlier generate is in flight: each ends with a synchronisation)
+  host->iters = 0; host->done = 0; host->err = 0u;
+  generate_begin_kernel<<<1, 256, 0, ctx->stream>>>(wsptr<int32_t>(ctx, ctx->ws.gen_count), wsptr<int32_t>(ctx, ctx->ws.nvalid),
+                                                    ctx->batch, ctx->n_nodes, done_word(ctx));
+  LAUNCH_CHECK();
+  int iters = 0;
+  CU(cudaEventRecord(ctx->ev0, ctx->stream));
+  for (; iters < limit; ++iters) {
+    for (int spins = 1; host->iters < iters - 1; ++spins) {
+      if ((spins & 0xfff) == 0) {
+        // the device has gone idle without a report: it failed
+        const cudaError_t q = cudaStreamQuery(ctx->stream);
+        if (q != cudaErrorNotReady && host->iters < iters - 1)
+          return fail(ctx, VADUSA_ECUDA, "generate: %s", q == cudaSuccess ? "an iteration was not reported" : cudaGetErrorString(q));
+      }
+    }
+    if (host->done >= ctx->batch) break;
+    const std::string iter_key = KeyBuilder("iteration").add(sp).add(out_tokens).add(max_new_tokens).add(ctx->batch)
+                                     .add(ctx->n_nodes).add(ctx->block_table).add(attention_splits(ctx, ctx->n_nodes)).add(ctx->fused_enabled).add(ctx->att_stream).k;
+    vadusa_status s = run_graphed(ctx, iter_key, [&]() -> vadusa_status {
+      vadusa_status s = DISPATCH(draft<float>(ctx, sp), draft<bf16>(ctx, sp));
+      if (s) return s;
+      s = DISPATCH(forward<float>(ctx, tv, nullptr, nullptr), forward<bf16>(ctx, tv, nullptr, nullptr));
+      if (s) return s;
+      return DISPATCH(accept_commit<float>(ctx, sp, nullptr, none, out_tokens, max_new_tokens, max_new_tokens, ctx->h_pinned),
+                      accept_commit<bf16>(ctx, sp, nullptr, none, out_tokens, max_new_tokens, max_new_tokens, ctx->h_pinned));
+    });
+    if (s) return s;
+    ctx->ctx_bound += ctx->tree_max_depth + 1;
+    ctx->ctx_lo += 1;
+  }
+  CU(cudaEventRecord(ctx->ev1, ctx->stream));
+  generate_end_kernel<<<1, 256, 0, ctx->stream>>>(wsptr<int32_t>(ctx, ctx->ws.gen_count), err_word(ctx), ctx->batch, max_new_tokens,
+                                                  out_len, host);
+  LAUNCH_CHECK();
+  if (h_out_tokens)
+    CU(cudaMemcpyAsync(h_out_tokens, out_tokens, (size_t)ctx->batch * max_new_tokens * 4, cudaMemcpyDeviceToHost, ctx->stream));
+  CU(cudaStreamSynchronize(ctx->stream));
+  int64_t total = 0;
+  for (int b = 0; b < ctx->batch; ++b) {
+    const int32_t g = host->gen[b];
+    total += g;
+    if (h_out_len) h_out_len[b] = g > max_new_tokens ? max_new_tokens : g;
+    if (ctx->h_ctx_exact) ctx->h_ctx[b] += g;               // (every committed token is counted in both)
+  }
+  if (h_stats) {
+    float ms = 0.f;
+    CU(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
+    h_stats->iterations = iters;
+    h_stats->tokens_generated = total;
+    h_stats->elapsed_ms = ms;
+    h_stats->kernel_launches = ctx->launches - launches0;
+  }
+  ctx->have_draft = ctx->have_verify = false;
+  return error_of(ctx, host->err);
 }
 
 }  // namespace
@@ -1256,8 +1495,9 @@ vadusa_status vadusa_init(const vadusa_weights* weights, const vadusa_config* cf
   if (vadusa_status s = set_kernel_attributes(ctx)) return s;
   CU(cudaEventCreate(&ctx->ev0));
   CU(cudaEventCreate(&ctx->ev1));
-  CU(cudaEventCreateWithFlags(&ctx->ev_poll, cudaEventDisableTiming));
-  CU(cudaMallocHost(&ctx->h_pinned, 4 * sizeof(int32_t)));
+  for (int i = 0; i < 2; ++i) CU(cudaEventCreateWithFlags(&ctx->ev_up[i], cudaEventDisableTiming));
+  CU(cudaMallocHost(&ctx->h_pinned, (kHostWords + cfg->max_batch) * sizeof(int32_t)));
+  CU(cudaMallocHost(&ctx->up, 2 * kUpHalf));
   CU(cudaMemsetAsync(ctx->wsp, 0, ctx->ws.tokens, ctx->stream));     // scalars, per-sequence state, trees
   CU(cudaMemsetAsync(ctx->wsp + ctx->ws.acc_stats, 0, 2ull * kStatDepth * kStatTopk * 8, ctx->stream));
   CU(cudaMemsetAsync(ctx->wsp + ctx->ws.f_sync, 0, 256, ctx->stream));
@@ -1281,8 +1521,9 @@ vadusa_status vadusa_destroy(vadusa_ctx* ctx) {
   if (!ctx) return VADUSA_EINVAL;
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
   if (ctx->ev1) cudaEventDestroy(ctx->ev1);
-  if (ctx->ev_poll) cudaEventDestroy(ctx->ev_poll);
+  for (int i = 0; i < 2; ++i) if (ctx->ev_up[i]) cudaEventDestroy(ctx->ev_up[i]);
   if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
+  if (ctx->up) cudaFreeHost(ctx->up);
   for (auto& r : ctx->prof) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
   for (auto& kv : ctx->graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   delete ctx;
@@ -1341,13 +1582,17 @@ vadusa_status vadusa_set_tree(vadusa_ctx* ctx, int32_t n_nodes, const int32_t* h
       if (has[n]) inner[(size_t)s * VADUSA_MAX_TREE_NODES + k++] = n;
     max_inner = k > max_inner ? k : max_inner;
   }
-  const size_t n4 = (size_t)copies * n_nodes * sizeof(int32_t);
-  CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_parent, h_parent, n4, cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_rank, h_rank, n4, cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_depth, depth.data(), n4, cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_inner, inner.data(), inner.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.tree_anc, anc.data(), (size_t)copies * n_nodes * 16, cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
+  // one staged copy: parent, depth, rank [copies][n_nodes], the lists of inner nodes, the ancestor words
+  const size_t nn = (size_t)copies * n_nodes;
+  std::vector<char> pack(nn * 12 + inner.size() * 4 + 16 + nn * 16);
+  const size_t at_anc = (nn * 12 + inner.size() * 4 + 15) & ~(size_t)15;
+  memcpy(pack.data(), h_parent, nn * 4);
+  memcpy(pack.data() + nn * 4, depth.data(), nn * 4);
+  memcpy(pack.data() + nn * 8, h_rank, nn * 4);
+  memcpy(pack.data() + nn * 12, inner.data(), inner.size() * 4);
+  memcpy(pack.data() + at_anc, anc.data(), nn * 16);
+  if (vadusa_status s = upload(ctx, ctx->wsp + ctx->ws.tree, pack.data(), at_anc + nn * 16)) return s;
+  ctx->tree_copies = copies;
   ctx->n_nodes = n_nodes;
   ctx->tree_per_seq = per_sequence ? 1 : 0;
   ctx->max_rank_used = max_rank;
@@ -1367,25 +1612,26 @@ vadusa_status vadusa_begin(vadusa_ctx* ctx, int32_t batch, const int32_t* block_
   ctx->batch = batch;
   ctx->block_table = block_table;
   ctx->have_draft = ctx->have_verify = false;
-  CU(cudaMemsetAsync(ctx->wsp + ctx->ws.scalars, 0, 256, ctx->stream));
-  CU(cudaMemsetAsync(ctx->wsp + ctx->ws.f_sync, 0, 256, ctx->stream));
-  CU(cudaMemsetAsync(ctx->wsp + ctx->ws.att_cnt, 0, 2 * kAsGrid * 4, ctx->stream));
-  CU(cudaMemsetAsync(ctx->wsp + ctx->ws.gen_count, 0, batch * 4, ctx->stream));
   ctx->ctx_bound = 0;
-  ctx->ctx_lo = 0;
+  ctx->h_ctx.assign(batch, 0);
+  ctx->h_ctx_exact = true;
   if (h_ctx_len) {
     for (int b = 0; b < batch; ++b) {
       if (h_ctx_len[b] < 0 || h_ctx_len[b] > (int64_t)ctx->cfg.max_blocks_per_seq * 64)
         return fail(ctx, VADUSA_EINVAL, "context length of sequence %d out of range", b);
       if (h_ctx_len[b] > ctx->ctx_bound) ctx->ctx_bound = h_ctx_len[b];
+      ctx->h_ctx[b] = h_ctx_len[b];
     }
-    ctx->ctx_lo = ctx->ctx_bound;
-    CU(cudaMemcpyAsync(ctx->wsp + ctx->ws.ctx_len, h_ctx_len, batch * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
-  } else {
-    CU(cudaMemsetAsync(ctx->wsp + ctx->ws.ctx_len, 0, batch * 4, ctx->stream));
+    if (vadusa_status s = upload(ctx, ctx->wsp + ctx->ws.ctx_len, h_ctx_len, batch * 4)) return s;
   }
-  return set_active(ctx, ctx->n_nodes);
+  ctx->ctx_lo = ctx->ctx_bound;
+  // one launch for everything a new batch clears
+  begin_kernel<<<1, 256, 0, ctx->stream>>>(wsptr<uint32_t>(ctx, ctx->ws.scalars), wsptr<uint32_t>(ctx, ctx->ws.f_sync),
+                                           wsptr<uint32_t>(ctx, ctx->ws.att_cnt), 2 * kAsGrid, wsptr<int32_t>(ctx, ctx->ws.gen_count),
+                                           h_ctx_len ? nullptr : wsptr<int32_t>(ctx, ctx->ws.ctx_len),
+                                           wsptr<int32_t>(ctx, ctx->ws.nvalid), batch, ctx->n_nodes);
+  LAUNCH_CHECK();
+  return VADUSA_OK;
 }
 
 vadusa_status vadusa_prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h_len, int32_t stride) {
@@ -1484,78 +1730,14 @@ vadusa_status vadusa_accept_and_commit(vadusa_ctx* ctx, const vadusa_sampling* s
   if (s) return s;
   ctx->ctx_bound += ctx->tree_max_depth + 1;
   ctx->ctx_lo += 1;
+  ctx->h_ctx_exact = false;
   ctx->have_verify = ctx->have_draft = false;
   return VADUSA_OK;
 }
 
 vadusa_status vadusa_generate(vadusa_ctx* ctx, const vadusa_sampling* sampling, int32_t max_new_tokens,
                               int32_t max_iters, int32_t* out_tokens, int32_t* out_len, vadusa_stats* h_stats) {
-  if (vadusa_status s = need_batch(ctx)) return s;
-  if (ctx->n_nodes == 0 || ctx->tree_per_seq) return fail(ctx, VADUSA_ESTATE, "generate needs a shared tree template");
-  if (max_new_tokens < 1) return fail(ctx, VADUSA_EINVAL, "max_new_tokens must be positive");
-  SamplingDev sp;
-  if (vadusa_status s = sampling_dev(ctx, sampling, &sp)) return s;
-  const int64_t launches0 = ctx->launches;
-  const int limit = max_iters > 0 ? max_iters : max_new_tokens;
-  const TreeView tv = tree_of(ctx, false);
-  AcceptOut none{nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr};
-  CU(cudaMemsetAsync(ctx->wsp + ctx->ws.gen_count, 0, ctx->batch * 4, ctx->stream));
-  CU(cudaMemsetAsync(done_word(ctx), 0, 4, ctx->stream));
-  if (vadusa_status s = set_active(ctx, ctx->n_nodes)) return s;
-  ctx->h_pinned[0] = 0;
-  bool poll_pending = false;
-  int iters = 0;
-  CU(cudaEventRecord(ctx->ev0, ctx->stream));
-  for (; iters < limit; ++iters) {
-    if (poll_pending && cudaEventQuery(ctx->ev_poll) == cudaSuccess) {
-      poll_pending = false;
-      if (ctx->h_pinned[0] >= ctx->batch) break;
-    }
-    // stay at most sixteen iterations ahead of the device: when the next poll is due and the last one has not come
-    // back, wait for it (iterations enqueued behind the end of the last sequence find nothing to do, but cost time)
-    if (poll_pending && (iters & 7) == 7) {
-      CU(cudaEventSynchronize(ctx->ev_poll));
-      poll_pending = false;
-      if (ctx->h_pinned[0] >= ctx->batch) break;
-    }
-    const std::string iter_key = KeyBuilder("iteration").add(sp).add(out_tokens).add(max_new_tokens).add(ctx->batch)
-                                     .add(ctx->n_nodes).add(ctx->block_table).add(attention_splits(ctx, ctx->n_nodes)).add(ctx->fused_enabled).add(ctx->att_stream).k;
-    vadusa_status s = run_graphed(ctx, iter_key, [&]() -> vadusa_status {
-      vadusa_status s = DISPATCH(draft<float>(ctx, sp), draft<bf16>(ctx, sp));
-      if (s) return s;
-      s = DISPATCH(forward<float>(ctx, tv, nullptr, nullptr), forward<bf16>(ctx, tv, nullptr, nullptr));
-      if (s) return s;
-      return DISPATCH(accept_commit<float>(ctx, sp, nullptr, none, out_tokens, max_new_tokens, max_new_tokens),
-                      accept_commit<bf16>(ctx, sp, nullptr, none, out_tokens, max_new_tokens, max_new_tokens));
-    });
-    if (s) return s;
-    ctx->ctx_bound += ctx->tree_max_depth + 1;
-    ctx->ctx_lo += 1;
-    if (!poll_pending && (iters & 7) == 7) {
-      CU(cudaMemcpyAsync(ctx->h_pinned, done_word(ctx), 4, cudaMemcpyDeviceToHost, ctx->stream));
-      CU(cudaEventRecord(ctx->ev_poll, ctx->stream));
-      poll_pending = true;
-    }
-  }
-  CU(cudaEventRecord(ctx->ev1, ctx->stream));
-  // lengths: min(gen_count, max_new_tokens) — computed on the host after the final sync
-  std::vector<int32_t> gen(ctx->batch);
-  CU(cudaMemcpyAsync(gen.data(), ctx->wsp + ctx->ws.gen_count, ctx->batch * 4, cudaMemcpyDeviceToHost, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
-  int64_t total = 0;
-  for (int b = 0; b < ctx->batch; ++b) { total += gen[b]; gen[b] = gen[b] > max_new_tokens ? max_new_tokens : gen[b]; }
-  if (out_len) CU(cudaMemcpyAsync(out_len, gen.data(), ctx->batch * 4, cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
-  if (h_stats) {
-    float ms = 0.f;
-    CU(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
-    h_stats->iterations = iters;
-    h_stats->tokens_generated = total;
-    h_stats->elapsed_ms = ms;
-    h_stats->kernel_launches = ctx->launches - launches0;
-  }
-  ctx->have_draft = ctx->have_verify = false;
-  return device_errors(ctx);
+  return run_generate(ctx, sampling, max_new_tokens, max_iters, out_tokens, out_len, nullptr, nullptr, h_stats);
 }
 
 vadusa_status vadusa_generate_host(vadusa_ctx* ctx, const vadusa_sampling* sampling, int32_t batch,
@@ -1570,15 +1752,7 @@ vadusa_status vadusa_generate_host(vadusa_ctx* ctx, const vadusa_sampling* sampl
   if (s) return s;
   s = vadusa_prefill(ctx, h_tokens, h_len, stride);
   if (s) return s;
-  int32_t* d_out = wsptr<int32_t>(ctx, ctx->ws.gen_out);
-  int32_t* d_len = wsptr<int32_t>(ctx, ctx->ws.gen_len);
-  s = vadusa_generate(ctx, sampling, max_new_tokens, 0, d_out, d_len, h_stats);
-  if (s == VADUSA_OK) {
-    cudaMemcpyAsync(h_out_tokens, d_out, (size_t)batch * max_new_tokens * 4, cudaMemcpyDeviceToHost, ctx->stream);
-    cudaMemcpyAsync(h_out_len, d_len, (size_t)batch * 4, cudaMemcpyDeviceToHost, ctx->stream);
-  }
-  CU(cudaStreamSynchronize(ctx->stream));
-  return s;
+  return run_generate(ctx, sampling, max_new_tokens, 0, wsptr<int32_t>(ctx, ctx->ws.gen_out), nullptr, h_out_tokens, h_out_len, h_stats);
 }
 
 vadusa_status vadusa_get_lengths(vadusa_ctx* ctx, int32_t* h_ctx_len) {
@@ -1589,6 +1763,8 @@ vadusa_status vadusa_get_lengths(vadusa_ctx* ctx, int32_t* h_ctx_len) {
   long long longest = 0;
   for (int b = 0; b < ctx->batch; ++b) longest = h_ctx_len[b] > longest ? h_ctx_len[b] : longest;
   ctx->ctx_lo = ctx->ctx_bound = longest;                   // both estimates are exact again
+  ctx->h_ctx.assign(h_ctx_len, h_ctx_len + ctx->batch);
+  ctx->h_ctx_exact = true;
   return VADUSA_OK;
 }
 

@@ -100,10 +100,10 @@ struct WorkspaceLayout {
   int64_t ctx_len, nvalid, gen_count, commit_base, commit_nv, root;   // int32 [B]
   int64_t node_ok, node_top;             // int32 [B][128]: the node is among its parent's draws; its own first draw
   int64_t seq_order;                     // int32 [R]: rows by descending context length
-  int64_t tree_parent, tree_depth, tree_rank, tree_anc;       // [B*128] (anc: two uint64 per node)
-  int64_t tree_inner;                    // [B*128]: nodes that have children, -1 behind the last
+  int64_t tree;                          // trees of the batch, packed (vadusa_set_tree): parent, depth, rank [copies][nodes], the nodes
+                                         // that have children [copies][128] (-1 behind the last), two uint64 ancestor words per node
   int64_t chain_parent, chain_depth, chain_rank, chain_anc;   // [128]
-  int64_t tokens, stage_tokens;          // int32 [M]
+  int64_t tokens;                        // int32 [M]
   int64_t kv_row;                        // int64 [M]: element offset of the row's K slot (head 0) in a layer's pool, -1: none
   int64_t topk;                          // int32 [B][heads][k]
   int64_t x;                             // fp32 [M][d]
@@ -119,9 +119,8 @@ struct WorkspaceLayout {
   int64_t acc_stats;                     // uint64 [2][VADUSA_MAX_DEPTH][VADUSA_MAX_DRAFT_TOPK]: edges tested, edges accepted
   int64_t gen_out, gen_len;              // int32 [B][kGenHostCap], int32 [B] (vadusa_generate_host staging)
   // prefill: one row per prefix chunk of a pass (R = pass_rows)
-  int64_t pf_ctx_len, pf_nvalid, pf_seq, pf_last;   // int32 [R]: tokens before the chunk, its length, its sequence, sequence if last chunk else -1
+  int64_t pf_stage;                      // a pass's arrays, packed (PassArrays in api.cu)
   int64_t pf_block_table;                // int32 [R][max_blocks_per_seq]: the block-table row of the chunk's sequence
-  int64_t pf_pairs;                      // int2 [R]: rows that share an attention CTA during prefill (y < 0: a single chunk)
   // single-sequence pass in one persistent kernel: residual stream after the attention block, LayerNorm statistics
   // per (token, group of 64 features) of both residual buffers, counters of the exchanges between clusters
   int64_t f_xb, f_stats_a, f_stats_b, f_sync;    // fp32 [64][d], float2 [64][d/64] x 2, uint32 [64]
@@ -140,11 +139,10 @@ inline WorkspaceLayout workspace_layout(const vadusa_config* c) {
   w.node_ok = take(B * VADUSA_MAX_TREE_NODES * 4); w.node_top = take(B * VADUSA_MAX_TREE_NODES * 4);
   w.seq_order = take(R * 4);
   const int64_t T = VADUSA_MAX_TREE_NODES;
-  w.tree_parent = take(B * T * 4); w.tree_depth = take(B * T * 4); w.tree_rank = take(B * T * 4);
-  w.tree_anc = take(B * T * 16); w.tree_inner = take(B * T * 4);
+  w.tree = take(B * T * 32 + 16);
   w.chain_parent = take(T * 4); w.chain_depth = take(T * 4); w.chain_rank = take(T * 4);
   w.chain_anc = take(T * 16);
-  w.tokens = take(M * 4); w.stage_tokens = take(M * 4);
+  w.tokens = take(M * 4);
   w.kv_row = take(M * 8);
   w.topk = take(B * hd * c->draft_topk * 4);
   w.x = take(M * d * 4);
@@ -159,9 +157,8 @@ inline WorkspaceLayout workspace_layout(const vadusa_config* c) {
   w.ln_stats = take(kLnStatsBytes);
   w.acc_stats = take(2ll * VADUSA_MAX_DEPTH * VADUSA_MAX_DRAFT_TOPK * 8);
   w.gen_out = take(B * kGenHostCap * 4); w.gen_len = take(B * 4);
-  w.pf_ctx_len = take(R * 4); w.pf_nvalid = take(R * 4); w.pf_seq = take(R * 4); w.pf_last = take(R * 4);
+  w.pf_stage = take(R * 40 + M * 4);
   w.pf_block_table = take(R * (int64_t)c->max_blocks_per_seq * 4);
-  w.pf_pairs = take(R * 8);
   w.f_xb = take(64 * d * 4);
   w.f_stats_a = take(64 * (d / 64 + 1) * 8); w.f_stats_b = take(64 * (d / 64 + 1) * 8);
   w.f_sync = take(256);

@@ -53,13 +53,15 @@ vadusa_status run(unsigned char* scratch, const void* dw, const float* db, const
   int32_t* active = reinterpret_cast<int32_t*>(scratch + kStaticScratchBytes - 256);
   set_active_words<<<1, 64, 0, stream>>>(active, batch);
   EpiDraftHiddenFlat<T> eh{db, reinterpret_cast<const T*>(hstar), z, d, batch};
-  dim3 g1((heads * d + 63) / 64, (batch + 63) / 64, 1);
-  gemm_simt_kernel<T, EpiDraftHiddenFlat<T>><<<g1, 256, 0, stream>>>(
-      reinterpret_cast<const T*>(hstar), reinterpret_cast<const T*>(dw), batch, heads * d, d, 0, 0, eh);
+  // (batch <= 64: the few-token kernel)
+  const int mw = batch <= 4 ? 1 : batch <= 8 ? 2 : 4, nw = 4 / mw;
+  dim3 g1((heads * d + 4 * nw - 1) / (4 * nw), (batch + 4 * mw - 1) / (4 * mw), 1);
+  gemm_few_kernel<T, EpiDraftHiddenFlat<T>, false><<<g1, 128, 0, stream>>>(
+      reinterpret_cast<const T*>(hstar), reinterpret_cast<const T*>(dw), batch, heads * d, d, 0, 0, mw, eh, RowNorm{});
   EpiLogits el{logits, ld, (long long)batch * ld};
-  dim3 g2((ld + 63) / 64, (batch + 63) / 64, heads);
-  gemm_simt_kernel<T, EpiLogits><<<g2, 256, 0, stream>>>(z, reinterpret_cast<const T*>(du), batch, ld, d,
-                                                         (long long)batch * d, (long long)ld * d, el);
+  dim3 g2((ld + 4 * nw - 1) / (4 * nw), (batch + 4 * mw - 1) / (4 * mw), heads);
+  gemm_few_kernel<T, EpiLogits, false><<<g2, 128, 0, stream>>>(z, reinterpret_cast<const T*>(du), batch, ld, d,
+                                                               (long long)batch * d, (long long)ld * d, mw, el, RowNorm{});
   SamplingDev sp = {};
   sp.tau = 1; sp.temperature = 0.f; sp.inv_temperature = 1.f; sp.top_p = 1.f;
   sp.eos_masked = eos_masked ? 1 : 0; sp.eos_id = vocab - 1;
