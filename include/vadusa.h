@@ -324,7 +324,8 @@ vadusa_status vadusa_build_sparse_tree(const double *h_prob, int32_t depth, int3
  * lambda 0.8, learning rate 0.002, 40 warm-up steps).  The paper names no optimiser and no normalisation:
  * here every head's cross-entropy is averaged over the positions that have a target, the optimiser is Adam
  * (beta 0.9 / 0.999, eps 1e-8, no weight decay), and the learning rate rises linearly over the warm-up steps.
- * Not part of the decoding path: plain fp32 arithmetic on fp32 master copies of the heads kept in `state`
+ * Not part of the decoding path: fp32 master copies of the heads and fp32 arithmetic (products from operands cut
+ * into three bf16 parts, 24 significant bits, with fp32 sums), kept in `state`
  * (device memory owned by the caller, >= vadusa_fit_state_bytes(cfg, max_tokens), 256-byte aligned).
  * vadusa_fit_begin copies the heads from the weight blob; every vadusa_fit_step writes the updated heads
  * back INTO THE CALLER'S WEIGHT BLOB (tensors "draft<i>.w/.b/.u", in the model dtype), so the next

@@ -1107,20 +1107,23 @@ vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h
 
 // ---- draft-head fitting -------------------------------------------------------------------
 struct FitLayout {
-  int64_t W, b, U, n_params;               // fp32 masters, contiguous: [heads][d][d], [heads][d], [heads][vpad][d]
-  int64_t m, v, g;                         // Adam moments and gradients, same shape as the masters
-  int64_t hf, pre, z, dz, logits, ce, count, total;
+  int64_t W, U, b;                         // fp32 masters: [heads][d][d], [heads][vpad][d], [heads][d]
+  int64_t mW, vW, mU, vU, mb, vb;          // Adam moments, same shapes
+  int64_t Wp, Up;                          // parts of the masters, bf16 [3] of the same shapes
+  int64_t hf, hp, pre, zp, dl, dp, logits, ce, count, total;
 };
 FitLayout fit_layout(const vadusa_config* c, int max_tokens) {
   FitLayout f;
   const int64_t hd = c->n_draft_heads, d = c->d_model, vp = vpad(c), T = max_tokens;
   int64_t off = 0;
   auto take = [&](int64_t bytes) { int64_t o = off; off = align_up(off + bytes, 256); return o; };
-  f.n_params = hd * (d * d + d + vp * d);
-  f.W = take(f.n_params * 4); f.b = f.W + hd * d * d * 4; f.U = f.b + hd * d * 4;
-  f.m = take(f.n_params * 4); f.v = take(f.n_params * 4); f.g = take(f.n_params * 4);
-  f.hf = take(T * d * 4); f.pre = take(hd * T * d * 4); f.z = take(hd * T * d * 4); f.dz = take(hd * T * d * 4);
-  f.logits = take(hd * T * vp * 4); f.ce = take(hd * T * 4); f.count = take(hd * 4);
+  const int64_t nW = hd * d * d, nU = hd * vp * d, nb = hd * d;
+  f.W = take(nW * 4); f.U = take(nU * 4); f.b = take(nb * 4);
+  f.mW = take(nW * 4); f.vW = take(nW * 4); f.mU = take(nU * 4); f.vU = take(nU * 4); f.mb = take(nb * 4); f.vb = take(nb * 4);
+  f.Wp = take(nW * 6); f.Up = take(nU * 6);
+  f.hf = take(T * d * 4); f.hp = take(T * d * 6); f.pre = take(hd * T * d * 4); f.zp = take(hd * T * d * 6);
+  f.dl = take(hd * T * vp * 6); f.dp = take(hd * T * d * 6); f.logits = take(hd * T * vp * 4);
+  f.ce = take(hd * T * 4); f.count = take(hd * 4);
   f.total = off;
   return f;
 }
@@ -1129,70 +1132,73 @@ template <typename T>
 vadusa_status fit_begin(vadusa_ctx* ctx, const FitLayout& f) {
   const vadusa_config& c = ctx->cfg;
   const long long hd = c.n_draft_heads, d = c.d_model, vp = vpad(&c);
-  auto up = [&](const T* src, int64_t off, long long n) -> vadusa_status {
-    fit_to_f32_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(src, reinterpret_cast<float*>(ctx->fit + off), n);
+  auto up = [&](const T* src, int64_t off, int64_t parts, long long n) -> vadusa_status {
+    fit_masters_kernel<T><<<(unsigned)((n / 8 + 255) / 256), 256, 0, ctx->stream>>>(src, reinterpret_cast<float*>(ctx->fit + off),
+                                                                                   reinterpret_cast<bf16*>(ctx->fit + parts), n);
     LAUNCH_CHECK();
     return VADUSA_OK;
   };
-  if (vadusa_status s = up(as<T>(ctx->dw), f.W, hd * d * d)) return s;
-  if (vadusa_status s = up(as<T>(ctx->du), f.U, hd * vp * d)) return s;
+  if (vadusa_status s = up(as<T>(ctx->dw), f.W, f.Wp, hd * d * d)) return s;
+  if (vadusa_status s = up(as<T>(ctx->du), f.U, f.Up, hd * vp * d)) return s;
   CU(cudaMemcpyAsync(ctx->fit + f.b, ctx->db, (size_t)(hd * d * 4), cudaMemcpyDeviceToDevice, ctx->stream));
-  CU(cudaMemsetAsync(ctx->fit + f.m, 0, (size_t)(f.n_params * 4), ctx->stream));
-  CU(cudaMemsetAsync(ctx->fit + f.v, 0, (size_t)(f.n_params * 4), ctx->stream));
+  CU(cudaMemsetAsync(ctx->fit + f.mW, 0, (size_t)(f.Wp - f.mW), ctx->stream));
+  return VADUSA_OK;
+}
+
+// One product of a fitting step: C[r][c] = sum_k A(r, k) B(c, k) per head (fit_tc_kernel).
+struct FitOperand { const void* parts; int rows, cols, heads; };   // the array as it lies: [part][heads][rows][cols]
+template <int NA, int NB, bool AMN, bool BMN, typename Epi>
+vadusa_status fit_product(vadusa_ctx* ctx, const FitOperand& A, const FitOperand& B, int R, int C, int K, const Epi& epi) {
+  static unsigned long long attr_done = 0ull;              // per device, like launch_gemm_tc
+  const unsigned long long dev_bit = 1ull << (ctx->cfg.device & 63);
+  if (!(attr_done & dev_bit)) {
+    CU(cudaFuncSetAttribute(fit_tc_kernel<NA, NB, AMN, BMN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, FitCfg<NA, NB>::kSmem));
+    attr_done |= dev_bit;
+  }
+  const CUtensorMap *ma, *mb;
+  if (vadusa_status s = tensor_map(ctx, A.parts, A.rows, A.cols, AMN ? 64 : kFitTile, NA * A.heads, (long long)A.rows * A.cols, &ma)) return s;
+  if (vadusa_status s = tensor_map(ctx, B.parts, B.rows, B.cols, BMN ? 64 : kFitTile, NB * B.heads, (long long)B.rows * B.cols, &mb)) return s;
+  CU(launch_dependent(ctx, fit_tc_kernel<NA, NB, AMN, BMN, Epi>,
+                      dim3((C + kFitTile - 1) / kFitTile, (R + kFitTile - 1) / kFitTile, ctx->cfg.n_draft_heads), kFitThreads,
+                      FitCfg<NA, NB>::kSmem, *ma, *mb, R, C, K, A.heads, B.heads, epi, err_word(ctx)));
+  LAUNCH_CHECK();
   return VADUSA_OK;
 }
 
 template <typename T>
 vadusa_status fit_step(vadusa_ctx* ctx, const FitLayout& f, const T* hidden, const int32_t* targets, int Tn, float* loss_out) {
+  constexpr int NH = sizeof(T) == 2 ? 1 : 3;               // parts of the hidden states
   const vadusa_config& c = ctx->cfg;
   const int hd = c.n_draft_heads, d = c.d_model, vp = vpad(&c), V = c.vocab;
   auto P = [&](int64_t off) { return reinterpret_cast<float*>(ctx->fit + off); };
-  float *W = P(f.W), *b = P(f.b), *U = P(f.U), *gW = P(f.g), *gb = gW + (long long)hd * d * d, *gU = gb + (long long)hd * d;
-  float *hf = P(f.hf), *pre = P(f.pre), *z = P(f.z), *dz = P(f.dz), *lg = P(f.logits), *ce = P(f.ce);
+  auto H = [&](int64_t off) { return reinterpret_cast<bf16*>(ctx->fit + off); };
   int32_t* count = reinterpret_cast<int32_t*>(ctx->fit + f.count);
-  const long long hs = (long long)Tn * d, ls = (long long)Tn * vp;
-  cudaStream_t st = ctx->stream;
-  auto gemm = [&](const float* A, const float* B, float* C, int M, int N, int K, long long sam, long long sak, long long sbn,
-                  long long sbk, long long ldc, long long az, long long bz, long long cz) -> vadusa_status {
-    dim3 grid((N + 63) / 64, (M + 63) / 64, hd);
-    fit_gemm_kernel<<<grid, 256, 0, st>>>(A, B, C, M, N, K, sam, sak, sbn, sbk, ldc, az, bz, cz);
-    LAUNCH_CHECK();
-    return VADUSA_OK;
-  };
-  const unsigned eb = (unsigned)((hs + 255) / 256);
-  fit_to_f32_kernel<T><<<eb, 256, 0, st>>>(hidden, hf, hs);
-  LAUNCH_CHECK();
-  fit_count_kernel<<<1, 256, 0, st>>>(targets, Tn, hd, count);
-  LAUNCH_CHECK();
-  // forward: pre = h W^T (+ b), z = h + SiLU(pre), logits = z U^T
-  if (vadusa_status s = gemm(hf, W, pre, Tn, d, d, d, 1, d, 1, d, 0, (long long)d * d, hs)) return s;
-  fit_hidden_kernel<<<dim3(eb, hd), 256, 0, st>>>(pre, b, hf, z, Tn, d, hs);
-  LAUNCH_CHECK();
-  if (vadusa_status s = gemm(z, U, lg, Tn, vp, d, d, 1, d, 1, vp, hs, (long long)vp * d, ls)) return s;
-  // loss and d loss / d logits (over the logits)
-  fit_softmax_ce_kernel<<<dim3(Tn, hd), 256, 0, st>>>(lg, targets, count, Tn, hd, V, vp, ctx->fit_lambda, ce);
-  LAUNCH_CHECK();
-  fit_loss_kernel<<<1, 256, 0, st>>>(ce, count, Tn, hd, ctx->fit_lambda, loss_out);
-  LAUNCH_CHECK();
-  // backward: dU = dl^T z, dz = dl U, dpre = dz SiLU'(pre), dW = dpre^T h, db = column sums of dpre
-  if (vadusa_status s = gemm(lg, z, gU, vp, d, Tn, 1, vp, 1, d, d, ls, hs, (long long)vp * d)) return s;
-  if (vadusa_status s = gemm(lg, U, dz, Tn, d, vp, vp, 1, 1, d, d, ls, (long long)vp * d, hs)) return s;
-  fit_dpre_kernel<<<dim3(eb, hd), 256, 0, st>>>(dz, pre, hs, hs);
-  LAUNCH_CHECK();
-  if (vadusa_status s = gemm(dz, hf, gW, d, d, Tn, 1, d, 1, d, d, hs, 0, (long long)d * d)) return s;
-  fit_colsum_kernel<<<dim3((d + 255) / 256, hd), 256, 0, st>>>(dz, gb, Tn, d, hs);
-  LAUNCH_CHECK();
-  // update (Adam, linear warm-up), masters and the heads in the weight blob
+  const FitOperand h{H(f.hp), Tn, d, 1}, z{H(f.zp), Tn, d, hd}, dl{H(f.dl), Tn, vp, hd}, dpre{H(f.dp), Tn, d, hd}, W{H(f.Wp), d, d, hd},
+      U{H(f.Up), vp, d, hd};
   ctx->fit_step++;
   const float lr = ctx->fit_lr * fminf(1.0f, (float)ctx->fit_step / (float)(ctx->fit_warmup > 0 ? ctx->fit_warmup : 1));
   const float c1 = (float)(1.0 - pow(0.9, (double)ctx->fit_step)), c2 = (float)(1.0 - pow(0.999, (double)ctx->fit_step));
-  float *mW = P(f.m), *vW = P(f.v);
-  const long long nW = (long long)hd * d * d, nb = (long long)hd * d, nU = (long long)hd * vp * d;
-  fit_adam_kernel<T><<<(unsigned)((nW + 255) / 256), 256, 0, st>>>(W, gW, mW, vW, const_cast<T*>(as<T>(ctx->dw)), nW, lr, c1, c2);
+  const long long n = (long long)Tn * d;
+  CU(launch_dependent(ctx, fit_inputs_kernel<T>, dim3((unsigned)((n / 8 + 255) / 256) + 1), 256, 0, hidden, P(f.hf), H(f.hp), n, targets,
+                      Tn, hd, count));
   LAUNCH_CHECK();
-  fit_adam_kernel<float><<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(b, gb, mW + nW, vW + nW, const_cast<float*>(ctx->db), nb, lr, c1, c2);
+  // forward: pre = h W^T + b, z = h + SiLU(pre), logits = z U^T
+  const FitHidden eh{P(f.b), P(f.hf), P(f.pre), H(f.zp), Tn, d, hd};
+  if (vadusa_status s = fit_product<NH, 3, false, false>(ctx, h, W, Tn, d, d, eh)) return s;
+  if (vadusa_status s = fit_product<3, 3, false, false>(ctx, z, U, Tn, vp, d, FitStore{P(f.logits), Tn, vp})) return s;
+  // loss and d loss / d logits
+  CU(launch_dependent(ctx, fit_softmax_ce_kernel, dim3(Tn, hd), 256, 0, (const float*)P(f.logits), targets, (const int32_t*)count, Tn, hd, V,
+                      vp, ctx->fit_lambda, H(f.dl), P(f.ce)));
   LAUNCH_CHECK();
-  fit_adam_kernel<T><<<(unsigned)((nU + 255) / 256), 256, 0, st>>>(U, gU, mW + nW + nb, vW + nW + nb, const_cast<T*>(as<T>(ctx->du)), nU, lr, c1, c2);
+  // backward and update: dz = dl U, dpre = dz SiLU'(pre); then dU = dl^T z and dW = dpre^T h with Adam behind the sums
+  // (linear warm-up; masters, their parts, and the heads in the weight blob)
+  if (vadusa_status s = fit_product<3, 3, false, true>(ctx, dl, U, Tn, d, vp, FitDpre{P(f.pre), H(f.dp), Tn, d, hd})) return s;
+  const FitAdam<T> aU{P(f.U), P(f.mU), P(f.vU), const_cast<T*>(as<T>(ctx->du)), H(f.Up), vp, d, hd, lr, c1, c2};
+  if (vadusa_status s = fit_product<3, 3, true, true>(ctx, dl, z, vp, d, Tn, aU)) return s;
+  const FitAdam<T> aW{P(f.W), P(f.mW), P(f.vW), const_cast<T*>(as<T>(ctx->dw)), H(f.Wp), d, d, hd, lr, c1, c2};
+  if (vadusa_status s = fit_product<3, NH, true, true>(ctx, dpre, h, d, d, Tn, aW)) return s;
+  CU(launch_dependent(ctx, fit_bias_kernel, dim3((d + 31) / 32 + 1, hd), 1024, 0, (const bf16*)H(f.dp), Tn, d, hd, P(f.b), P(f.mb), P(f.vb),
+                      const_cast<float*>(ctx->db), lr, c1, c2, (const float*)P(f.ce), (const int32_t*)count, ctx->fit_lambda, loss_out));
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
