@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(kPfThreads, 2) prefill_attention_tc_kernel(
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(ring_ptr + kAttRingBytes + 1024 + 16 * (SK + SV) + 80);
   volatile int* s_abort = reinterpret_cast<volatile int*>(ring_ptr + kAttRingBytes + 1024 + 16 * (SK + SV) + 84);   // a wait of the softmax threads ran out
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  __shared__ int s_blk[kAttBlocks];           // block ids of the first pages
   const int h = blockIdx.x;
 
   if (tid == 0) {
@@ -96,31 +97,25 @@ __global__ void __launch_bounds__(kPfThreads, 2) prefill_attention_tc_kernel(
   float m_use = -INFINITY, l_run = 0.f;       // softmax threads: scaling maximum (log2 units) and sum of weights
 
   if (warp == 8) {
-    // ---- TMA producer (lane 0)
-    long long blk_mine[2] = {0, 0};
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int i = lane + 32 * r;
-      if (i < ntiles) {
-        const long long v = kv_block_of(block_table, geom, rA, i * kKvBlock, err);
-        blk_mine[r] = v < 0 ? 0 : v;
-      }
+    // ---- TMA producer (one lane)
+    for (int i = lane; i < min(ntiles, kAttBlocks); i += 32) {
+      const long long v = kv_block_of(block_table, geom, rA, i * kKvBlock, err);
+      s_blk[i] = v < 0 ? 0 : (int)v;          // flagged; stay inside the pool
     }
-    if (lane == 0 && ntiles > 0) {
+    __syncwarp();
+    if (elect_one() && ntiles > 0) {
       mbar_expect_tx(bar_q, 2 * kAttTileBytes);
       tma_load_3d(q_addr, &tmQ, bar_q, h * 64, rA * 64, 0);
       tma_load_3d(q_addr + kAttTileBytes, &tmQ, bar_q, h * 64, (rB >= 0 ? rB : rA) * 64, 0);
-    }
-    bool ok = true;
-    for (int i = 0; i < ntiles; ++i) {
-      long long blk;
-      if (i < 64) {
-        blk = __shfl_sync(0xffffffffu, (i < 32) ? blk_mine[0] : blk_mine[1], i & 31);
-      } else {
-        blk = kv_block_of(block_table, geom, rA, i * kKvBlock, err);
-        if (blk < 0) blk = 0;
-      }
-      if (lane == 0 && ok) {
+      bool ok = true;
+      for (int i = 0; i < ntiles && ok; ++i) {
+        long long blk;
+        if (i < kAttBlocks) {
+          blk = s_blk[i];
+        } else {
+          blk = kv_block_of(block_table, geom, rA, i * kKvBlock, err);
+          if (blk < 0) blk = 0;
+        }
         const int sk = i % SK, sv = i % SV;
         const int row = (int)((blk * 2 * geom.n_heads + h) * kKvBlock);
         if (i >= SK && !mbar_wait(empty_k0 + 8 * sk, ((i / SK) - 1) & 1, err)) {
@@ -137,8 +132,8 @@ __global__ void __launch_bounds__(kPfThreads, 2) prefill_attention_tc_kernel(
       }
     }
   } else if (warp == 9) {
-    // ---- P V issuer (lane 0)
-    if (lane == 0) {
+    // ---- P V issuer (one lane)
+    if (elect_one()) {
       constexpr uint32_t idesc_pv = umma_idesc_bf16(128, 64) | (1u << 16);     // B (V tile) is MN-major
       for (int i = 0; i < ntiles; ++i) {
         if (!mbar_wait(bar_p0 + 8 * (i % 3), (i / 3) & 1, err)) break;
@@ -156,8 +151,8 @@ __global__ void __launch_bounds__(kPfThreads, 2) prefill_attention_tc_kernel(
       }
     }
   } else if (warp == 10) {
-    // ---- Q K^T issuer (lane 0)
-    if (lane == 0) {
+    // ---- Q K^T issuer (one lane)
+    if (elect_one()) {
       constexpr uint32_t idesc_qk = umma_idesc_bf16(128, 64);
       bool ok = ntiles == 0 || mbar_wait(bar_q, 0, err);
       for (int i = 0; i < ntiles && ok; ++i) {

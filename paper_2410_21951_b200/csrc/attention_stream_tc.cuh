@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kAsThreads, 2) tree_attention_stream_kernel(
   volatile int* s_abort = reinterpret_cast<volatile int*>(holder_ptr + 1);   // a softmax wait ran out
   volatile int* s_flag = reinterpret_cast<volatile int*>(holder_ptr + 2);    // this CTA merges the item's parts
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int N = tree.n_nodes, H = geom.n_heads;
   // CTA c works on head c % H for group c / H: the H CTAs of a group walk the same pages of the same sequences at
   // the same time, so that what is in flight in DRAM at any moment are runs of H adjacent K (and V) tiles
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kAsThreads, 2) tree_attention_stream_kernel(
   } else if (warp == 5) {
     // ---- P V issuer (lane 0): O += P V as soon as the softmax threads have stored P; a segment's first product
     // overwrites the accumulator (the softmax threads read the previous segment's before they store these weights)
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc_pv = umma_idesc_bf16(128, 64) | (1u << 16);     // B (V tile) is MN-major
       bool ok = true;
       int g = 0;
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kAsThreads, 2) tree_attention_stream_kernel(
   } else if (warp == 6) {
     // ---- Q K^T issuer (lane 0): S = Q K^T into score buffer g % 3, up to three pages ahead of P V, also across
     // the end of a segment
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc_qk = umma_idesc_bf16(128, 64);
       bool ok = true;
       int g = 0, s = 0;

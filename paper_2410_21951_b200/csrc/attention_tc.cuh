@@ -25,7 +25,7 @@
 // K and V tiles have rings of their own: a K tile is free as soon as its Q K^T has completed, a V tile after
 // its P V.  "Scores ready", "weights ready" and "P V done" have one mbarrier per score buffer: a buffer's next
 // use cannot begin before the waiter of the current one has passed, so no parity wait can fall a round behind.
-// Warps: 0-3 softmax, warp 4 lane 0 TMA producer, warp 5 TMEM owner / P V issuer, warp 6 Q K^T issuer.
+// Warps: 0-3 softmax, warp 4 TMA producer, warp 5 TMEM owner / P V issuer, warp 6 Q K^T issuer.
 #pragma once
 #include "tc.cuh"
 
@@ -38,6 +38,7 @@ constexpr int kAttTileBytes = 64 * 64 * 2;                                   // 
 constexpr int kAttRingBytes = (kAttStagesK + kAttStagesV) * kAttTileBytes;   // 80 KB; also holds the 64x64 fp32 output exchange
 constexpr int kAttSmemBytes = 2 * kAttTileBytes /*Q, 128 rows*/ + kAttRingBytes + 1024 /*sums, maxima*/ +
                               1024 /*alignment*/ + 256 /*barriers*/;
+constexpr int kAttBlocks = 64;                                               // block ids kept in shared memory
 constexpr float kAttRescaleStep = 6.0f;                                      // log2 units
 
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
@@ -139,7 +140,8 @@ __global__ void __launch_bounds__(kAttThreads) tree_attention_tc_kernel(
                                                                // buffer, so that a phase parity is never one round behind
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(ring_ptr + kAttRingBytes + 1024 + 16 * (SK + SV) + 80);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  __shared__ int s_blk[kAttBlocks];           // block ids of the first pages
   const int h = blockIdx.x, split = blockIdx.z;
   const int N = tree.n_nodes;
 
@@ -171,35 +173,29 @@ __global__ void __launch_bounds__(kAttThreads) tree_attention_tc_kernel(
   float m_use = -INFINITY, l_run = 0.f;       // softmax threads: scaling maximum (log2 units) and partial sum
 
   if (warp == 4) {
-    // ---- TMA producer (lane 0); the block ids of this CTA's pages are fetched by the whole warp first
-    long long blk_mine[2] = {0, 0};
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int i = lane + 32 * r;
-      if (i < ntiles) {
-        const long long v = kv_block_of(block_table, geom, b, (p0 + i) * kKvBlock, err);
-        blk_mine[r] = v < 0 ? 0 : v;          // flagged; stay inside the pool
-      }
+    // ---- TMA producer (one lane); the block ids of this CTA's pages are fetched by the whole warp first
+    for (int i = lane; i < min(ntiles, kAttBlocks); i += 32) {
+      const long long v = kv_block_of(block_table, geom, b, (p0 + i) * kKvBlock, err);
+      s_blk[i] = v < 0 ? 0 : (int)v;          // flagged; stay inside the pool
     }
-    if (lane == 0 && ntiles > 0) {
+    __syncwarp();
+    if (elect_one() && ntiles > 0) {
       mbar_expect_tx(bar_q, 2 * kAttTileBytes);
       tma_load_3d(q_addr, &tmQ, bar_q, h * 64, b * N + node0, 0);
       tma_load_3d(q_addr + kAttTileBytes, &tmQ, bar_q, h * 64, b * N + node0, 0);      // the same rows again: lanes 64..127
-    }
-    bool ok = true;
-    for (int i = 0; i < ntiles; ++i) {
-      long long blk;
-      if (i < 64) {
-        blk = __shfl_sync(0xffffffffu, (i < 32) ? blk_mine[0] : blk_mine[1], i & 31);
-      } else {
-        blk = kv_block_of(block_table, geom, b, (p0 + i) * kKvBlock, err);
-        if (blk < 0) blk = 0;
-      }
-      if (lane == 0 && ok) {
+      bool ok = true;
+      for (int i = 0; i < ntiles && ok; ++i) {
+        long long blk;
+        if (i < kAttBlocks) {
+          blk = s_blk[i];
+        } else {
+          blk = kv_block_of(block_table, geom, b, (p0 + i) * kKvBlock, err);
+          if (blk < 0) blk = 0;
+        }
         const int sk = i % SK, sv = i % SV;
         const int row = (int)((blk * 2 * geom.n_heads + h) * kKvBlock);
         if (i >= SK && !mbar_wait(empty_k0 + 8 * sk, ((i / SK) - 1) & 1, err)) {
-          ok = false;                         // timed out (recorded): stop issuing, keep the warp converged
+          ok = false;                         // timed out (recorded): stop issuing
         } else {
           mbar_expect_tx(full_k0 + 8 * sk, kAttTileBytes);
           tma_load_3d(ring + sk * kAttTileBytes, &tmKV, full_k0 + 8 * sk, 0, row, layer);
@@ -212,8 +208,8 @@ __global__ void __launch_bounds__(kAttThreads) tree_attention_tc_kernel(
       }
     }
   } else if (warp == 5) {
-    // ---- P V issuer (lane 0): O += P(i) V(i) as soon as the softmax threads have stored P(i)
-    if (lane == 0) {
+    // ---- P V issuer (one lane): O += P(i) V(i) as soon as the softmax threads have stored P(i)
+    if (elect_one()) {
       constexpr uint32_t idesc_pv = umma_idesc_bf16(128, 64) | (1u << 16);     // B (V tile) is MN-major
       for (int i = 0; i < ntiles; ++i) {
         if (!mbar_wait(bar_p0 + 8 * (i % 3), (i / 3) & 1, err)) break;
@@ -231,8 +227,8 @@ __global__ void __launch_bounds__(kAttThreads) tree_attention_tc_kernel(
       }
     }
   } else if (warp == 6) {
-    // ---- Q K^T issuer (lane 0): S(i) = Q K(i)^T into score buffer i % 3, up to three pages ahead of P V
-    if (lane == 0) {
+    // ---- Q K^T issuer (one lane): S(i) = Q K(i)^T into score buffer i % 3, up to three pages ahead of P V
+    if (elect_one()) {
       constexpr uint32_t idesc_qk = umma_idesc_bf16(128, 64);
       bool ok = ntiles == 0 || mbar_wait(bar_q, 0, err);
       for (int i = 0; i < ntiles && ok; ++i) {

@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kFitThreads) fit_tc_kernel(const __grid_consta
   const uint32_t bars = base + S * Cfg::kStageBytes;             // full[S], empty[S], accumulator, tmem holder
   const uint32_t full0 = bars, empty0 = bars + 8 * S, accum = bars + 16 * S, holder = accum + 8;
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem_raw + (holder - smem_u32(smem_raw)));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, head = blockIdx.z;
+  const int warp = warp_index(), lane = threadIdx.x & 31, head = blockIdx.z;
   const int c0 = blockIdx.x * kFitTile, r0 = blockIdx.y * kFitTile, nk = (K + 63) / 64;
 
   if (threadIdx.x == 0) {
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kFitThreads) fit_tc_kernel(const __grid_consta
   grid_dep_wait();
   grid_dep_launch();
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     auto load = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, bool mn, int row0, int k0, int z) {
       if (mn) {
         tma_load_3d(dst, map, bar, row0, k0, z);
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kFitThreads) fit_tc_kernel(const __grid_consta
       for (int p = 0; p < NB; ++p) load(st + (NA + p) * kFitPart, &tmB, full0 + 8 * s, BMN, c0, 64 * i, p * b_heads + (b_heads > 1 ? head : 0));
     }
   }
-  if (warp == 1 && lane == 0) {
+  if (warp == 1 && elect_one()) {
     constexpr uint32_t idesc = umma_idesc_bf16(kFitTile, kFitTile) | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u);
     for (int i = 0; i < nk; ++i) {
       const int s = i % S;

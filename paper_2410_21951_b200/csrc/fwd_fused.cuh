@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kFfThreads, 1) fused_forward_kernel(
   int* s_pageblk = reinterpret_cast<int*>(misc_p + 768);               // [kFfMaxPages] pool row of each of this CTA's pages
   long long* s_kvrow = reinterpret_cast<long long*>(misc_p + 896);     // [TPO] K slot of this CTA's tokens (head 0), or -1
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int rank = (int)cluster_rank();
   const int c = (int)blockIdx.x / CS;                    // cluster = head
   const int NC = (int)gridDim.x / CS;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kFfThreads, 1) fused_forward_kernel(
       s_pageblk[lane] = (int)((blk < 0 ? 0 : blk) * 2 * a.geom.n_heads + c) * kKvBlock;
     }
     __syncwarp();
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       // slot of item `seq`: waits until the item that used it before has been consumed; arms the barrier
       auto acquire = [&](int seq, uint32_t bytes) -> uint32_t {
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kFfThreads, 1) fused_forward_kernel(
     // =========================================================== MMA issuer
     grid_dep_wait();
     plan();
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t id128 = umma_idesc_bf16(128, 128), id64 = umma_idesc_bf16(128, 64);
       constexpr uint32_t id_pv = umma_idesc_bf16(128, 64) | (1u << 16);        // B (V tile) is MN-major
       const uint32_t acc = tmem + kFfColAcc;

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
   const uint32_t full0 = bars, empty0 = bars + 8 * S, accum_bar = bars + 16 * S, holder = bars + 16 * S + 8;
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(ring_ptr + ring_bytes + 16 * S + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * kGemmRowsW, m0 = blockIdx.y * TN;
   const int zb = blockIdx.z / ksplit, ks = blockIdx.z % ksplit;
   const int chunk0 = ks * chunks_per_split, nchunks = chunks_per_split;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *holder_ptr;
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     // ---- TMA producer
     const int pre = nchunks < S ? nchunks : S;
     for (int i = 0; i < pre; ++i) {                      // weights do not depend on the upstream kernel
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
       ln_operand<TN>(ln, M, nchunks * ksplit * kGemmBK, chunk0 * kGemmBK, base + kWBytes, Cfg::kStageBytes);
     __syncthreads();
   }
-  if (warp == 1 && lane == 0) {
+  if (warp == 1 && elect_one()) {
     // ---- MMA issuer
     constexpr uint32_t idesc = umma_idesc_bf16(kGemmRowsW, TN < 16 ? 16 : TN);
     // the token operand is requested only after the upstream grid has finished: wait for that first, so that the

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
   const uint32_t full0 = bars, empty0 = bars + 8 * S, accum_bar = bars + 16 * S, holder = bars + 16 * S + 8;
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(ring_ptr + kRing + 16 * S + 8);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();                  // 0: leader
   const int n0 = blockIdx.x * kGemmRowsW, m0 = blockIdx.y * TN;
 
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem = *holder_ptr;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     // ---- TMA producer (both CTAs): own weight rows, own half of the token tile
     const int pre = nchunks < S ? nchunks : S;
     for (int i = 0; i < pre; ++i) {                      // weights do not depend on the upstream kernel
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
       tma_load_3d_pair(base + s * Cfg::kStageBytes + kWBytes, &tmX, fb, i * kGemmBK, m0 + (int)rank * (TN / 2), 0);
     }
   }
-  if (warp == 1 && lane == 0 && rank == 0) {
+  if (warp == 1 && rank == 0 && elect_one()) {
     // ---- MMA issuer (leader only): 256 features x TN tokens per instruction
     constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
     for (int i = 0; i < nchunks; ++i) {
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kGemmP2Threads, 1) gemm_tc2p_kernel(const __gr
   const uint32_t full0 = bars, empty0 = bars + 8 * S, accf0 = bars + 16 * S, acce0 = accf0 + 16, holder = acce0 + 16;
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(ring_ptr + kRing + 16 * S + 32);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();                  // 0: leader
   const int pair = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
   const int nfp = N / (2 * kGemmRowsW);                  // feature pairs per token tile
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kGemmP2Threads, 1) gemm_tc2p_kernel(const __gr
   const uint32_t tmem = *holder_ptr;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer (both CTAs): own 128 weight rows, own half of the token tile; one chunk counter over all tiles
       bool waited = false, ok = true;
       long long g = 0;
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kGemmP2Threads, 1) gemm_tc2p_kernel(const __gr
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       // ---- MMA issuer (leader only): 256 features x 256 tokens per instruction, accumulator k & 1
       constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
       bool ok = true;

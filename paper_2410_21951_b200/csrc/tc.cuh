@@ -61,6 +61,17 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   return false;
 }
 
+// The warp's index as a value the compiler knows to be the same in all lanes, and one elected lane of a converged warp.
+// A role of one thread is entered through these: tcgen05 and TMA instructions take their operands from uniform registers,
+// and behind a branch on threadIdx alone the issuing thread was held 100-125 cycles by every MMA (at 4096 tokens the
+// first feed-forward product took 31.9 us, 25.5 with the elected lane; the second at 2048 tokens 23.7 and 21.2).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // TMA: 3-D tiled load global -> shared, completion counted in bytes on an mbarrier.
 // c0 is the innermost coordinate (its byte offset must be a multiple of 16).
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
