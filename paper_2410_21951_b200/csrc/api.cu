@@ -60,6 +60,7 @@ struct vadusa_ctx {
   int pf_tap_stride = 0;
   int pf_tiles = 0;           // > 0 while a prefill pass runs: attention CTAs of the pass (pairs of chunks), listed in pf_pairs
   const int2* pf_pairs = nullptr;
+  bool in_prefill = false;    // a prefill pass: the context of its later chunks is written by the pass itself
   int att_stream = 0;         // batches: attention as one persistent kernel over the stream of K/V pages (0: one CTA per head and sequence)
   int fused_enabled = 0;      // single-sequence passes run as one persistent kernel (0: no, 1: yes, 6 / 8: with that cluster size)
   int fused_clusters = -1;    // clusters of that kernel that can be resident at once on this device (-1: not asked yet)
@@ -571,7 +572,7 @@ vadusa_status attention(vadusa_ctx* ctx, const T* q, const T* pool, const TreeVi
     PROF(ctx, K_ATTENTION);
     CU(launch_dependent(ctx, kern, dim3(c.n_heads, ctx->batch, (tv.n_nodes + ng - 1) / ng), 256, att_simt_smem(dh), q, pool, ctx->block_table,
                         (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.ctx_len), (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.nvalid),
-                        tv, g, c.d_model, scale, out, err_word(ctx)));
+                        tv, g, c.d_model, scale, ctx->in_prefill ? 0 : 1, out, err_word(ctx)));
     LAUNCH_CHECK();
     return VADUSA_OK;
   };
@@ -651,7 +652,7 @@ vadusa_status attention(vadusa_ctx* ctx, const T* q, const T* pool, const TreeVi
                             (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.ctx_len),
                             (const int32_t*)wsptr<int32_t>(ctx, ctx->ws.nvalid),
                             (const int32_t*)(ctx->batch > 1 ? wsptr<int32_t>(ctx, ctx->ws.seq_order) : nullptr), tv, g, c.d_model,
-                            scale * 1.4426950408889634f, splits, reinterpret_cast<bf16*>(out),
+                            scale * 1.4426950408889634f, splits, ctx->in_prefill ? 0 : 1, reinterpret_cast<bf16*>(out),
                             wsptr<float>(ctx, ctx->ws.att_xch), err_word(ctx)));
       LAUNCH_CHECK();
       return VADUSA_OK;
@@ -1079,9 +1080,11 @@ vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h
       RowsView view(ctx, rows, d_table, ctx->ws.pf_stage + (int64_t)pa.ctx(), ctx->ws.pf_stage + (int64_t)pa.nvalid());
       const PrefillTail tail{ends, tail_tiles, reinterpret_cast<const int2*>(dev + pa.tail_pairs()), dp(pa.tail_m())};
       ctx->pf_tiles = tiles;
+      ctx->in_prefill = true;
       ctx->pf_pairs = reinterpret_cast<const int2*>(dev + pa.pairs());
       const vadusa_status s = forward<T>(ctx, tv, dp(pa.tokens()), nullptr, whole ? nullptr : &tail);
       ctx->pf_tiles = 0;
+      ctx->in_prefill = false;
       if (s) return s;
     }
     if (ends > 0) {

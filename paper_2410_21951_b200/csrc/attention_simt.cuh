@@ -29,7 +29,8 @@ template <typename T, int DH, int NG>
 __global__ void __launch_bounds__(256) tree_attention_simt_kernel(
     const T* q, const T* pool, const int32_t* __restrict__ block_table,
     const int32_t* ctx_len, const int32_t* nvalid, TreeView tree, KvGeom geom,
-    int d_model, float scale, T* __restrict__ out, uint32_t* err) {
+    int d_model, float scale, int ahead /*rows inside the context may be read before the upstream kernel ends: not while prefilling*/,
+    T* __restrict__ out, uint32_t* err) {
   constexpr int R = DH / 32;
   __shared__ float4 Qs[NG][DH / 4];
   __shared__ float4 Ps[8][NG][8];             // a warp's weights: [node][32 keys]
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(256) tree_attention_simt_kernel(
       kr[i] = t0 + u / U < total ? att_ld4<T>(Kg + 4 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
-  const bool early = 32 * warp + 32 <= S && nv > 0;
+  const bool early = ahead && 32 * warp + 32 <= S && nv > 0;
   if (early) fetch_keys(32 * warp);
   unsigned long long alo[NG], ahi[NG];
 #pragma unroll
