@@ -376,15 +376,15 @@ vadusa_status launch_gemm_tc(vadusa_ctx* ctx, int cls, const void* X, const void
 }
 
 // Many-token product on CTA pairs (256 features x TN tokens per pair, no K split).
-template <int TN, int ST, typename Epi>
+template <int TN, int ST, int KB, typename Epi>
 vadusa_status launch_gemm_tc2(vadusa_ctx* ctx, int cls, const void* X, const void* W, int w_rows, int M, int N, int K,
                               const Epi& epi) {
-  using Cfg = GemmTc2Cfg<TN, ST>;
+  using Cfg = GemmTc2Cfg<TN, ST, KB>;
   static unsigned long long attr_done = 0ull;              // per device, like launch_gemm_tc
   const unsigned long long dev_bit = 1ull << (ctx->cfg.device & 63);
   if (!(attr_done & dev_bit)) {
-    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
-    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, Epi>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
+    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, Epi>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     attr_done |= dev_bit;
   }
   const CUtensorMap *mw, *mx;
@@ -402,7 +402,7 @@ vadusa_status launch_gemm_tc2(vadusa_ctx* ctx, int cls, const void* X, const voi
   at[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at; lc.numAttrs = 2;
   PROF(ctx, cls);
-  CU(cudaLaunchKernelEx(&lc, gemm_tc2_kernel<TN, ST, Epi>, *mw, *mx, M, N, K / kGemmBK, epi, err_word(ctx)));
+  CU(cudaLaunchKernelEx(&lc, gemm_tc2_kernel<TN, ST, KB, Epi>, *mw, *mx, M, N, K / (kGemmBK * KB), epi, err_word(ctx)));
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
@@ -481,23 +481,30 @@ bool gemm_tc_ln(vadusa_ctx* ctx, int cls, const float* x, const float* g, const 
 template <typename Epi>
 vadusa_status gemm_tc(vadusa_ctx* ctx, int cls, const void* X, const void* W, int w_rows, int M, int N, int K,
                       int batches, long long x_z, long long w_z, const Epi& epi) {
-  // token tile: as narrow as the token count allows for weight streaming; 256 for the tensor-bound shapes
-  // when that still gives every SM a CTA pair, else 128
   const int ntiles_n = (N + kGemmRowsW - 1) / kGemmRowsW;
-  // tensor-bound shapes whose features come in whole pairs of tiles: CTA pairs, when they fill the SMs.  Of
-  // the 256-token tile (two CTAs per SM) and the 128-token tile (two per SM with four stages when all CTAs are
-  // resident at once, else three per SM with three stages) the one whose last wave is fuller; ties to the wider.
-  if (M > 512 && batches == 1 && N % (2 * kGemmRowsW) == 0) {
-    // at least two full rounds of 256 x 256 tiles per pair: resident pairs whose epilogue runs under the next tile
-    if ((N / (2 * kGemmRowsW)) * ((M + 255) / 256) >= 148) return launch_gemm_tc2p(ctx, cls, X, W, w_rows, M, N, K, epi);
-    auto fill = [](int ctas, int slots) { return (double)ctas / (double)(((ctas + slots - 1) / slots) * slots); };
-    const int c256 = ntiles_n * ((M + 255) / 256), c128 = ntiles_n * ((M + 127) / 128);
-    const double f256 = c256 >= 128 ? fill(c256, 296) : 0.0;
-    const double f128 = c128 >= 128 ? fill(c128, c128 <= 296 ? 296 : 444) : 0.0;
-    if (f256 > 0.0 && f256 >= f128) return launch_gemm_tc2<256, 3>(ctx, cls, X, W, w_rows, M, N, K, epi);
-    if (f128 > 0.0 && c128 <= 296) return launch_gemm_tc2<128, 4>(ctx, cls, X, W, w_rows, M, N, K, epi);
-    if (f128 > 0.0) return launch_gemm_tc2<128, 3>(ctx, cls, X, W, w_rows, M, N, K, epi);
+  // More than 64 tokens and features in whole pairs of tiles: CTA pairs.  While a tile width gives at most one CTA per SM, the
+  // narrowest such tile with the deepest ring of two-chunk stages (every CTA streams operands, latency decides); then
+  // 128-token tiles with two or three CTAs per SM, whose epilogues hide behind one another's main loops; beyond three
+  // full SMs' worth, resident pairs that walk 256 x 256 tiles.  32-token tiles read every weight M / 32 times: up to 72 CTAs, and
+  // up to a full device where the weights are not the wider operand (N <= K).  Measured with weights from DRAM, us:
+  //   512 tokens: q/k/v 13.8 -> 8.0, out 8.7 -> 4.9, FFN1 13.9 -> 8.6, FFN2 11.4 -> 11.1 (before: one CTA per tile, K split)
+  //   2048 tokens: FFN1 17.8 -> 15.9, FFN2 21.4 -> 16.1; 1344 tokens: out 17.2 -> 8.0, FFN2 25.8 -> 15.4
+  // Few tokens against a long K (second feed-forward matrix) stay with the K split below: 7.9 us at 128 tokens, 10.5 as pairs.
+  if (M > 64 && batches == 1 && N % (2 * kGemmRowsW) == 0 && !(M <= 128 && K > 2 * N)) {
+    auto ctas = [&](int tn) { return ntiles_n * ((M + tn - 1) / tn); };
+    const bool two = K % (2 * kGemmBK) == 0;             // stages of two chunks
+    if (two && ctas(32) <= (N <= K ? 148 : 72)) {
+      if (ctas(32) <= 72 || K > 1024) return launch_gemm_tc2<32, 5, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
+      return launch_gemm_tc2<32, 3, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    }
+    if (two && ctas(64) <= 148) return launch_gemm_tc2<64, 4, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    if (two && ctas(128) <= 148) return launch_gemm_tc2<128, 4, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    if (!two && ctas(64) <= 296) return launch_gemm_tc2<64, 5, 1>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    if (ctas(128) <= 296) return launch_gemm_tc2<128, 4, 1>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    if (ctas(128) <= 444) return launch_gemm_tc2<128, 3, 1>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    return launch_gemm_tc2p(ctx, cls, X, W, w_rows, M, N, K, epi);
   }
+  // token tile: as narrow as the token count allows for weight streaming; 256 where that still gives every SM a CTA pair
   int tn = M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : M <= 1024 ? 128 : 256;
   if (tn == 256 && ntiles_n * ((M + 255) / 256) * batches < 200) tn = 128;
   const int tiles = ((N + kGemmRowsW - 1) / kGemmRowsW) * ((M + tn - 1) / tn) * batches;

@@ -17,11 +17,13 @@
 
 namespace vadusa {
 
-// ST stages of 16 KB of weights + TN/2 token rows.  Several CTAs (of different pairs) share an SM, so that one's
-// epilogue overlaps another's main loop: two with <256, 3> (TMEM: 2 x 256 columns) and <128, 4>, three with <128, 3>.
-template <int TN, int ST> struct GemmTc2Cfg {
+// ST stages of KB chunks (64 columns of K each) of 128 weight rows + TN/2 token rows.  KB = 2: a stage's wait, fence and
+// commit serve eight instructions instead of four.  Small rings leave room for several CTAs (of different pairs) on an SM, so
+// that one's epilogue overlaps another's main loop.
+template <int TN, int ST, int KB> struct GemmTc2Cfg {
   static constexpr int kXHalfBytes = (TN / 2) * kGemmBK * 2;
-  static constexpr int kStageBytes = kGemmRowsW * kGemmBK * 2 + kXHalfBytes;
+  static constexpr int kChunkBytes = kGemmRowsW * kGemmBK * 2 + kXHalfBytes;
+  static constexpr int kStageBytes = KB * kChunkBytes;
   static constexpr int kStages = ST;
   static constexpr int kTmemCols = TN;
   static constexpr int kSmem = kStages * kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
@@ -66,11 +68,11 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
                ::"r"(bar), "h"(both) : "memory");
 }
 
-template <int TN, int ST, typename Epi>
+template <int TN, int ST, int KB, typename Epi>
 __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmW,
                                                        const __grid_constant__ CUtensorMap tmX /*box: TN/2 rows*/,
-                                                       int M, int N, int nchunks, Epi epi, uint32_t* err) {
-  using Cfg = GemmTc2Cfg<TN, ST>;
+                                                       int M, int N, int nsteps /*K / (64 KB)*/, Epi epi, uint32_t* err) {
+  using Cfg = GemmTc2Cfg<TN, ST, KB>;
   constexpr int S = Cfg::kStages;
   constexpr uint32_t kWBytes = kGemmRowsW * kGemmBK * 2, kXBytes = Cfg::kXHalfBytes;
   constexpr int kRing = S * Cfg::kStageBytes;
@@ -101,35 +103,47 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
 
   if (warp == 0 && elect_one()) {
     // ---- TMA producer (both CTAs): own weight rows, own half of the token tile
-    const int pre = nchunks < S ? nchunks : S;
+    auto load_w = [&](int i, int s, uint32_t fb) {
+#pragma unroll
+      for (int j = 0; j < KB; ++j)
+        tma_load_3d_pair(base + s * Cfg::kStageBytes + j * Cfg::kChunkBytes, &tmW, fb, (i * KB + j) * kGemmBK, n0, 0);
+    };
+    auto load_x = [&](int i, int s, uint32_t fb) {
+#pragma unroll
+      for (int j = 0; j < KB; ++j)
+        tma_load_3d_pair(base + s * Cfg::kStageBytes + j * Cfg::kChunkBytes + kWBytes, &tmX, fb, (i * KB + j) * kGemmBK,
+                         m0 + (int)rank * (TN / 2), 0);
+    };
+    const int pre = nsteps < S ? nsteps : S;
     for (int i = 0; i < pre; ++i) {                      // weights do not depend on the upstream kernel
-      if (rank == 0) mbar_expect_tx(full0 + 8 * i, 2 * (kWBytes + kXBytes));
-      tma_load_3d_pair(base + i * Cfg::kStageBytes, &tmW, map_to_cta(full0 + 8 * i, 0), i * kGemmBK, n0, 0);
+      if (rank == 0) mbar_expect_tx(full0 + 8 * i, 2 * Cfg::kStageBytes);
+      load_w(i, i, map_to_cta(full0 + 8 * i, 0));
     }
     grid_dep_wait();
-    for (int i = 0; i < pre; ++i)
-      tma_load_3d_pair(base + i * Cfg::kStageBytes + kWBytes, &tmX, map_to_cta(full0 + 8 * i, 0), i * kGemmBK,
-                       m0 + (int)rank * (TN / 2), 0);
-    for (int i = pre; i < nchunks; ++i) {
+    for (int i = 0; i < pre; ++i) load_x(i, i, map_to_cta(full0 + 8 * i, 0));
+    for (int i = pre; i < nsteps; ++i) {
       const int s = i % S;
       if (!mbar_wait(empty0 + 8 * s, ((i / S) - 1) & 1, err)) break;
-      if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * (kWBytes + kXBytes));
+      if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * Cfg::kStageBytes);
       const uint32_t fb = map_to_cta(full0 + 8 * s, 0);
-      tma_load_3d_pair(base + s * Cfg::kStageBytes, &tmW, fb, i * kGemmBK, n0, 0);
-      tma_load_3d_pair(base + s * Cfg::kStageBytes + kWBytes, &tmX, fb, i * kGemmBK, m0 + (int)rank * (TN / 2), 0);
+      load_w(i, s, fb);
+      load_x(i, s, fb);
     }
   }
   if (warp == 1 && rank == 0 && elect_one()) {
     // ---- MMA issuer (leader only): 256 features x TN tokens per instruction
     constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
-    for (int i = 0; i < nchunks; ++i) {
+    for (int i = 0; i < nsteps; ++i) {
       const int s = i % S;
       if (!mbar_wait(full0 + 8 * s, (i / S) & 1, err)) break;
       tc_fence_after();
-      const uint32_t wa = base + s * Cfg::kStageBytes, xa = wa + kWBytes;
 #pragma unroll
-      for (int k = 0; k < kGemmBK / 16; ++k)
-        umma_bf16_pair(tmem, umma_desc_k_sw128(wa + 32 * k), umma_desc_k_sw128(xa + 32 * k), idesc, (i | k) != 0);
+      for (int j = 0; j < KB; ++j) {
+        const uint32_t wa = base + s * Cfg::kStageBytes + j * Cfg::kChunkBytes, xa = wa + kWBytes;
+#pragma unroll
+        for (int k = 0; k < kGemmBK / 16; ++k)
+          umma_bf16_pair(tmem, umma_desc_k_sw128(wa + 32 * k), umma_desc_k_sw128(xa + 32 * k), idesc, (i | j | k) != 0);
+      }
       umma_commit_pair(empty0 + 8 * s);                  // the stage is reusable in both CTAs
     }
     umma_commit_pair(accum_bar);                         // both accumulators complete
