@@ -1076,6 +1076,15 @@ vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h
       }
       r += pair ? 2 : 1;
     }
+    // longest contexts first: their CTAs would otherwise be the last to start (80 000 tokens in ragged prefixes: 39.6 -> 37.0 ms)
+    auto longest_first = [&](int32_t* pairs, int n) {
+      struct Pair { int32_t x, y; };
+      Pair* q = reinterpret_cast<Pair*>(pairs);
+      const int32_t* cl = at(pa.ctx());
+      std::stable_sort(q, q + n, [&](const Pair& u, const Pair& v) { return cl[u.x] > cl[v.x]; });
+    };
+    longest_first(at(pa.pairs()), tiles);
+    longest_first(at(pa.tail_pairs()), tail_tiles);
     char* dev = ctx->wsp + ctx->ws.pf_stage;
     if (vadusa_status s = upload(ctx, dev, pack.data(), pack.size())) return s;
     auto dp = [&](size_t off) { return reinterpret_cast<int32_t*>(dev + off); };
