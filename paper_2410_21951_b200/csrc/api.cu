@@ -1076,8 +1076,11 @@ vadusa_status prefill(vadusa_ctx* ctx, const int32_t* h_tokens, const int32_t* h
       }
       r += pair ? 2 : 1;
     }
-    // longest contexts first: their CTAs would otherwise be the last to start (80 000 tokens in ragged prefixes: 39.6 -> 37.0 ms)
+    // Longest contexts first: their CTAs would otherwise be the last to start (80 000 tokens in ragged prefixes: 39.6 -> 37.0 ms).
+    // Not where all CTAs run at once: the first few share SMs that the projection left free, and these should be the short
+    // ones (one prefix of 325 tokens: 11.8 us a launch in order of position, 15.5 sorted)
     auto longest_first = [&](int32_t* pairs, int n) {
+      if (ctx->cfg.n_heads * n <= 2 * 148) return;
       struct Pair { int32_t x, y; };
       Pair* q = reinterpret_cast<Pair*>(pairs);
       const int32_t* cl = at(pa.ctx());
