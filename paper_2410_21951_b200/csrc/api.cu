@@ -676,8 +676,8 @@ vadusa_status layernorm(vadusa_ctx* ctx, const float* x, const float* g, const f
   const int d = ctx->cfg.d_model;
   const bool by_warp = rows >= 64 && d % 128 == 0 && d <= 2048;   // many rows: one warp per row
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(by_warp ? (rows + 7) / 8 : rows);
-  lc.blockDim = dim3(256);
+  lc.gridDim = dim3(by_warp ? (rows + 3) / 4 : rows);
+  lc.blockDim = dim3(by_warp ? 128 : 256);
   lc.stream = ctx->stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;       // the kernel calls griddepcontrol.wait
@@ -1244,6 +1244,14 @@ vadusa_status set_kernel_attributes(vadusa_ctx* ctx) {
   CU(cudaFuncSetAttribute(commit_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
   CU(cudaFuncSetAttribute(commit_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
   CU(cudaFuncSetAttribute(draft_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 24576 * (int)sizeof(float)));
+  // the small kernels between the products too: an SM that keeps its carve-out takes the next kernel's CTAs beside them
+  const auto carve = cudaFuncAttributePreferredSharedMemoryCarveout;
+  CU(cudaFuncSetAttribute(layernorm_rows_kernel<float>, carve, cudaSharedmemCarveoutMaxShared));
+  CU(cudaFuncSetAttribute(layernorm_rows_kernel<bf16>, carve, cudaSharedmemCarveoutMaxShared));
+  CU(cudaFuncSetAttribute(layernorm_kernel<bf16>, carve, cudaSharedmemCarveoutMaxShared));
+  CU(cudaFuncSetAttribute(tree_embed_kernel<bf16>, carve, cudaSharedmemCarveoutMaxShared));
+  CU(cudaFuncSetAttribute(commit_kernel<bf16>, carve, cudaSharedmemCarveoutMaxShared));
+  CU(cudaFuncSetAttribute(draft_select_kernel, carve, cudaSharedmemCarveoutMaxShared));
   // ask for the largest shared-memory carve-out so that several CTAs fit on an SM
   CU(cudaFuncSetAttribute(tree_attention_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   CU(cudaFuncSetAttribute(tree_attention_stream_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));

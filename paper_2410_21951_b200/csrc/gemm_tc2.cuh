@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
   if (warp == 1 && rank == 0 && elect_one()) {
     // ---- MMA issuer (leader only): 256 features x TN tokens per instruction
     constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
+    grid_dep_wait();                                     // the bounded waits below time this kernel's own pipeline only
     for (int i = 0; i < nsteps; ++i) {
       const int s = i % S;
       if (!mbar_wait(full0 + 8 * s, (i / S) & 1, err)) break;
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(kGemmP2Threads, 1) gemm_tc2p_kernel(const __gr
       constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
       bool ok = true;
       long long g = 0;
+      grid_dep_wait();                                   // (as above)
       for (int k = 0; k < my_tiles && ok; ++k) {
         const int b = k & 1;
         // both CTAs' epilogue warps have read what tile k - 2 left in this accumulator
