@@ -49,7 +49,6 @@ struct vadusa_ctx {
   int n_nodes = 0;            // current tree size (0: none set)
   int tree_per_seq = 0;
   int tree_copies = 1;        // trees in the workspace's tree area (packed: see vadusa_set_tree)
-  int max_rank_used = 0;
   int tree_max_depth = 0;
   int tree_inner = 0;         // most nodes with children of any of the trees
   // draft-head fitting (vadusa_fit_*): the caller's state buffer and the schedule
@@ -1582,7 +1581,7 @@ vadusa_status vadusa_set_tree(vadusa_ctx* ctx, int32_t n_nodes, const int32_t* h
   std::vector<int32_t> depth((size_t)copies * n_nodes);
   std::vector<unsigned long long> anc((size_t)copies * n_nodes * 2);
   std::vector<int32_t> inner((size_t)copies * VADUSA_MAX_TREE_NODES, -1);
-  int max_rank = 0, max_depth = 0, max_inner = 0;
+  int max_depth = 0, max_inner = 0;
   for (int s = 0; s < copies; ++s) {
     const int32_t* par = h_parent + (size_t)s * n_nodes;
     const int32_t* rnk = h_rank + (size_t)s * n_nodes;
@@ -1608,7 +1607,6 @@ vadusa_status vadusa_set_tree(vadusa_ctx* ctx, int32_t n_nodes, const int32_t* h
         if (par[n] < par[n - 1] || (par[n] == par[n - 1] && rnk[n] <= rnk[n - 1]))
           return fail(ctx, VADUSA_EINVAL, "node %d: nodes of one depth must be in rank-path order", n);
       }
-      max_rank = rnk[n] > max_rank ? rnk[n] : max_rank;
       max_depth = dep[n] > max_depth ? dep[n] : max_depth;
     }
     bool has[VADUSA_MAX_TREE_NODES] = {false};
@@ -1631,7 +1629,6 @@ vadusa_status vadusa_set_tree(vadusa_ctx* ctx, int32_t n_nodes, const int32_t* h
   ctx->tree_copies = copies;
   ctx->n_nodes = n_nodes;
   ctx->tree_per_seq = per_sequence ? 1 : 0;
-  ctx->max_rank_used = max_rank;
   ctx->tree_max_depth = max_depth;
   ctx->tree_inner = max_inner > 0 ? max_inner : 1;
   ctx->have_draft = ctx->have_verify = false;

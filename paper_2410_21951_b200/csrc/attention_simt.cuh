@@ -20,7 +20,7 @@ template <> __device__ __forceinline__ float4 att_ld4<bf16>(const bf16* p) {
 // the lanes turn to the features and add the weighted V rows), each with running maxima and sums of its own; they are
 // merged once at the end.  A short context is one chunk per warp: three dependent loads and one block barrier (17 us before,
 // with a block per head that staged 64-key pages one after another).  Rows read straight into the lanes that own them
-// touch 32 lines per load: 9 us for 16 nodes over 120-200 keys; through shared memory see the figure at the launch.
+// touch 32 lines per load: 9 us for 16 nodes over 120-200 keys, about 4 us through shared memory.
 // NG = 4 while the blocks are few, 8 when they fill the device several times (half the K/V reads).
 // Dynamic shared memory: att_simt_smem(DH).
 inline int att_simt_smem(int dh) { return 8 * 32 * (dh + 4) * 4; }

@@ -113,8 +113,8 @@ struct SelectScratch {
 // 1025 tokens).  The first interval is what the peak alone decides: below max + T ln((1 - top_p) Z / vocab) all tokens
 // together weigh less than 1 - top_p.
 //   val[]   in: logits (EOS masked) in shared memory;  prob[] out: exp((val - max) / T)
-// On return token j is inside iff bits(val[j]) > lo, where *exact tells that the tokens at *hi (the only ones in
-// (lo, hi]) are tied and *above their mass ahead; without ties everything above lo is inside.
+// On return token j is inside iff bits(val[j]) > lo, where `tied` tells that the tokens at hi (the only ones in
+// (lo, hi]) are tied and `above` is their mass ahead; without ties everything above lo is inside.
 struct Nucleus { uint32_t lo, hi; float above, limit; bool tied; };
 
 __device__ Nucleus nucleus_of(const float* val, float* prob, int vocab, const SamplingDev& sp, SelectScratch& sc) {
