@@ -24,6 +24,8 @@
 // order), and the normalised, scaled and shifted slice is written as bf16 straight into the
 // operand's swizzled shared-memory layout.
 #pragma once
+#include <type_traits>
+
 #include "tc.cuh"
 
 namespace vadusa {
@@ -238,21 +240,38 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
     cluster_sync_all();                                  // release / acquire: the peers' tiles are visible
     const int per = TN / ksplit;
     const int n4 = (threadIdx.x & 31) * 4;
-    for (int t = ks * per + warp; t < (ks + 1) * per; t += 4) {
-      // (one block, so that the epilogue's own loads can be issued beside the peers')
-      if (m0 + t < M && n0 + n4 < N) {                                        // N is a multiple of 4
-        const float* a = part + tile_id * (TN * kGemmRowsW) + t * kGemmRowsW + n4;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 pv[kGemmMaxSplit];
+    // A warp finishes TT tokens at a time, all of whose partial rows are requested before the first is used: with eight slices
+    // of a 64-token tile one round trip to L2 instead of two (q/k/v 9.0 -> 8.5 us, FFN1 8.9 -> 8.4 inside a batch-1 step).
+    // (One block, so that the epilogue's own loads can be issued beside the peers'.)
+    auto merge = [&](auto peers_c, auto tokens_c) {
+      constexpr int PP = decltype(peers_c)::value, TT = decltype(tokens_c)::value;
+      if (n0 + n4 >= N) return;                                               // N is a multiple of 4
+      const int t1 = min((ks + 1) * per, M - m0);
+      for (int t0 = ks * per + warp; t0 < t1; t0 += 4 * TT) {
+        float4 pv[TT][PP];
 #pragma unroll
-        for (int peer = 0; peer < kGemmMaxSplit; ++peer)
-          if (peer < ksplit) pv[peer] = __ldcg(reinterpret_cast<const float4*>(a + (long long)peer * (TN * kGemmRowsW)));
+        for (int u = 0; u < TT; ++u) {
+          const float* a = part + tile_id * (TN * kGemmRowsW) + (t0 + 4 * u) * kGemmRowsW + n4;
 #pragma unroll
-        for (int peer = 0; peer < kGemmMaxSplit; ++peer)
-          if (peer < ksplit) { acc.x += pv[peer].x; acc.y += pv[peer].y; acc.z += pv[peer].z; acc.w += pv[peer].w; }
-        epi.vec4(zb, m0 + t, n0 + n4, acc);
+          for (int peer = 0; peer < PP; ++peer)
+            if (peer < ksplit && t0 + 4 * u < t1) pv[u][peer] = __ldcg(reinterpret_cast<const float4*>(a + (long long)peer * (TN * kGemmRowsW)));
+        }
+#pragma unroll
+        for (int u = 0; u < TT; ++u) {
+          if (t0 + 4 * u < t1) {
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int peer = 0; peer < PP; ++peer)
+              if (peer < ksplit) { acc.x += pv[u][peer].x; acc.y += pv[u][peer].y; acc.z += pv[u][peer].z; acc.w += pv[u][peer].w; }
+            epi.vec4(zb, m0 + t0 + 4 * u, n0 + n4, acc);
+          }
+        }
       }
-    }
+    };
+    using std::integral_constant;
+    if (ksplit > 8) merge(integral_constant<int, kGemmMaxSplit>{}, integral_constant<int, 1>{});
+    else if (ksplit > 4) merge(integral_constant<int, 8>{}, integral_constant<int, 2>{});
+    else merge(integral_constant<int, 4>{}, integral_constant<int, 4>{});
   }
   tc_fence_before();
   __syncthreads();
