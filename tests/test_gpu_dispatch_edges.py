@@ -12,10 +12,10 @@ from harness import TOL, read_kv, tokens_with_phonemes
 pytestmark = pytest.mark.gpu
 
 
-def _prefill_rows_match(dtype, chunks, last, check, nodes=64):
+def _prefill_rows_match(dtype, chunks, last, check, nodes=64, d_ffn=1024):
     """`chunks` sequences of one chunk each (the last of `last` tokens) in one pass; K/V rows of the checked ones."""
     import paper_2410_21951_b200 as P
-    wl = W.toy_workload(dtype=dtype, d_model=256, n_heads=4, d_ffn=1024, vocab=203, tree_nodes=16, tree_caps=(6, 3, 2),
+    wl = W.toy_workload(dtype=dtype, d_model=256, n_heads=4, d_ffn=d_ffn, vocab=203, tree_nodes=16, tree_caps=(6, 3, 2),
                         batch=chunks, index=31)
     w = W.make_weights(wl.shape, wl.seed())
     model = O.Model.from_shape(wl.shape, w)
@@ -43,6 +43,12 @@ def _prefill_rows_match(dtype, chunks, last, check, nodes=64):
 @pytest.mark.parametrize("chunks,last", [(2, 64), (3, 1), (5, 37), (17, 64), (33, 5), (65, 64), (98, 33), (114, 64), (130, 9)])
 def test_bf16_products_of_many_tokens(chunks, last):
     _prefill_rows_match("bf16", chunks, last, sorted({0, chunks // 2, chunks - 1}))
+
+
+# up to 64 tokens the K slices of a product are merged by the tokens of a tile: 2, 4, 8 and 16 slices, tiles full or not
+@pytest.mark.parametrize("tokens,d_ffn", [(2, 1024), (15, 512), (16, 1024), (17, 512), (31, 1024), (33, 512), (63, 1024), (64, 512)])
+def test_bf16_split_products_of_few_tokens(tokens, d_ffn):
+    _prefill_rows_match("bf16", 1, tokens, [0], nodes=tokens, d_ffn=d_ffn)
 
 
 # the few-token product kernel serves up to 128 rows of a pass, the tile kernel beyond
