@@ -27,6 +27,8 @@
 // use cannot begin before the waiter of the current one has passed, so no parity wait can fall a round behind.
 // Warps: 0-3 softmax, warp 4 TMA producer, warp 5 TMEM owner / P V issuer, warp 6 Q K^T issuer.
 #pragma once
+#include <type_traits>
+
 #include "tc.cuh"
 
 namespace vadusa {
@@ -446,42 +448,50 @@ __global__ void __launch_bounds__(kAttThreads, 2) tree_attention_tc_kernel(
       if (oh == 0) { mine[64 * 64 + orow] = l_run; mine[64 * 64 + 64 + orow] = m_use; }
     }
     cluster_sync_all();                        // release / acquire: the peers' slots are visible
-    // CTA `split` finishes nodes [split*per_n, (split+1)*per_n): 16 threads per node, four consecutive
-    // features each
+    // CTA `split` finishes nodes [split*per_n, (split+1)*per_n): 16 threads per node, four consecutive features each.  All of a
+    // thread's nodes (one with eight splits, two with four, four with two) are requested before the first is merged: one
+    // round trip to L2 instead of up to four (batch 8, two splits: 14.4 -> 12.9 us per launch).
     const float* first = xch + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * splits * kSlot;
-    const int per_n = 64 / splits;
-    if (tid < 128) {
-      const int e4 = (tid & 15) * 4;
-      for (int n = split * per_n + (tid >> 4); n < (split + 1) * per_n; n += 8) {
-        float mm[8], ll[8];
-        float4 oo[8];
-        float M = -INFINITY;
+    auto merge = [&](auto splits_c) {
+      constexpr int PP = decltype(splits_c)::value, TT = 8 / PP;
+      const int e4 = (tid & 15) * 4, n = split * (64 / PP) + (tid >> 4);
+      float mm[TT][PP], ll[TT][PP];
+      float4 oo[TT][PP];
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < splits) {
-            const float* sl = first + (long long)p * kSlot;
-            mm[p] = __ldcg(sl + 64 * 64 + 64 + n);
-            ll[p] = __ldcg(sl + 64 * 64 + n);
-            oo[p] = __ldcg(reinterpret_cast<const float4*>(sl + n * 64 + e4));
-            M = fmaxf(M, mm[p]);
-          }
-        float L = 0.f;
+      for (int u = 0; u < TT; ++u)
+#pragma unroll
+        for (int p = 0; p < PP; ++p) {
+          const float* sl = first + (long long)p * kSlot;
+          mm[u][p] = __ldcg(sl + 64 * 64 + 64 + n + 8 * u);
+          ll[u][p] = __ldcg(sl + 64 * 64 + n + 8 * u);
+          oo[u][p] = __ldcg(reinterpret_cast<const float4*>(sl + (n + 8 * u) * 64 + e4));
+        }
+#pragma unroll
+      for (int u = 0; u < TT; ++u) {
+        float M = -INFINITY, L = 0.f;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < splits) {
-            const float w = (mm[p] == -INFINITY) ? 0.f : exp2f(mm[p] - M);
-            L = fmaf(ll[p], w, L);
-            o.x = fmaf(oo[p].x, w, o.x); o.y = fmaf(oo[p].y, w, o.y); o.z = fmaf(oo[p].z, w, o.z); o.w = fmaf(oo[p].w, w, o.w);
-          }
-        if (node0 + n < N) {
-          const float inv = (node0 + n < nv && L > 0.f) ? 1.f / L : 0.f;
+        for (int p = 0; p < PP; ++p) M = fmaxf(M, mm[u][p]);
+#pragma unroll
+        for (int p = 0; p < PP; ++p) {
+          const float w = (mm[u][p] == -INFINITY) ? 0.f : exp2f(mm[u][p] - M);
+          L = fmaf(ll[u][p], w, L);
+          o.x = fmaf(oo[u][p].x, w, o.x); o.y = fmaf(oo[u][p].y, w, o.y); o.z = fmaf(oo[u][p].z, w, o.z); o.w = fmaf(oo[u][p].w, w, o.w);
+        }
+        const int node = node0 + n + 8 * u;
+        if (node < N) {
+          const float inv = (node < nv && L > 0.f) ? 1.f / L : 0.f;
           uint2 v;
           v.x = pack_bf16(o.x * inv, o.y * inv);
           v.y = pack_bf16(o.z * inv, o.w * inv);
-          *reinterpret_cast<uint2*>(out + ((long long)b * N + node0 + n) * d_model + h * 64 + e4) = v;
+          *reinterpret_cast<uint2*>(out + ((long long)b * N + node) * d_model + h * 64 + e4) = v;
         }
       }
+    };
+    if (tid < 128) {
+      if (splits == 8) merge(std::integral_constant<int, 8>{});
+      else if (splits == 4) merge(std::integral_constant<int, 4>{});
+      else merge(std::integral_constant<int, 2>{});
     }
   }
 }
