@@ -377,8 +377,11 @@ vadusa_status launch_gemm_tc(vadusa_ctx* ctx, int cls, const void* X, const void
 // Many-token product on CTA pairs (256 features x TN tokens per pair, no K split).
 template <int TN, int ST, int KB, typename Epi>
 vadusa_status launch_gemm_tc2(vadusa_ctx* ctx, int cls, const void* X, const void* W, int w_rows, int M, int N, int K,
-                              const Epi& epi) {
+                              int slices, const Epi& epi) {
   using Cfg = GemmTc2Cfg<TN, ST, KB>;
+  // whole stages; and all CTAs that fit on an SM have room in its tensor memory, so that no pair ever waits for another's
+  constexpr int kPerSm = 227 * 1024 / (Cfg::kSmem + 1024), kAccCols = 512 / kPerSm < 256 ? 512 / kPerSm : 256;
+  while (slices > 1 && (slices * TN > kAccCols || K / (kGemmBK * KB) % slices)) slices /= 2;
   static unsigned long long attr_done = 0ull;              // per device, like launch_gemm_tc
   const unsigned long long dev_bit = 1ull << (ctx->cfg.device & 63);
   if (!(attr_done & dev_bit)) {
@@ -401,7 +404,7 @@ vadusa_status launch_gemm_tc2(vadusa_ctx* ctx, int cls, const void* X, const voi
   at[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at; lc.numAttrs = 2;
   PROF(ctx, cls);
-  CU(cudaLaunchKernelEx(&lc, gemm_tc2_kernel<TN, ST, KB, Epi>, *mw, *mx, M, N, K / (kGemmBK * KB), epi, err_word(ctx)));
+  CU(cudaLaunchKernelEx(&lc, gemm_tc2_kernel<TN, ST, KB, Epi>, *mw, *mx, M, N, K / (kGemmBK * KB), slices, epi, err_word(ctx)));
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
@@ -491,16 +494,20 @@ vadusa_status gemm_tc(vadusa_ctx* ctx, int cls, const void* X, const void* W, in
   // Few tokens against a long K (second feed-forward matrix) stay with the K split below: 7.9 us at 128 tokens, 10.5 as pairs.
   if (M > 64 && batches == 1 && N % (2 * kGemmRowsW) == 0 && !(M <= 128 && K > 2 * N)) {
     auto ctas = [&](int tn) { return ntiles_n * ((M + tn - 1) / tn); };
+    // Accumulators: one; for a prefix, whose rows every later token reads, one per K slice that a single-CTA product of 128-token
+    // tiles would be split into (shorter chains of truncating additions: the rows are the split form's to the bit).  One prefix
+    // of 325 tokens 668 -> 726 us a call; the same in a batch-8 step would be 3.00 -> 3.19 ms.
+    const int slices = !ctx->in_prefill || (M > 512 && ctas(128) >= 128) ? 1 : gemm_ksplit(ctas(128), K / kGemmBK, 128);
     const bool two = K % (2 * kGemmBK) == 0;             // stages of two chunks
     if (two && ctas(32) <= (N <= K ? 148 : 72)) {
-      if (ctas(32) <= 72 || K > 1024) return launch_gemm_tc2<32, 5, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
-      return launch_gemm_tc2<32, 3, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
+      if (ctas(32) <= 72 || K > 1024) return launch_gemm_tc2<32, 5, 2>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
+      return launch_gemm_tc2<32, 3, 2>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
     }
-    if (two && ctas(64) <= 148) return launch_gemm_tc2<64, 4, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
-    if (two && ctas(128) <= 148) return launch_gemm_tc2<128, 4, 2>(ctx, cls, X, W, w_rows, M, N, K, epi);
-    if (!two && ctas(64) <= 296) return launch_gemm_tc2<64, 5, 1>(ctx, cls, X, W, w_rows, M, N, K, epi);
-    if (ctas(128) <= 296) return launch_gemm_tc2<128, 4, 1>(ctx, cls, X, W, w_rows, M, N, K, epi);
-    if (ctas(128) <= 444) return launch_gemm_tc2<128, 3, 1>(ctx, cls, X, W, w_rows, M, N, K, epi);
+    if (two && ctas(64) <= 148) return launch_gemm_tc2<64, 4, 2>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
+    if (two && ctas(128) <= 148) return launch_gemm_tc2<128, 4, 2>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
+    if (!two && ctas(64) <= 296) return launch_gemm_tc2<64, 5, 1>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
+    if (ctas(128) <= 296) return launch_gemm_tc2<128, 4, 1>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
+    if (ctas(128) <= 444) return launch_gemm_tc2<128, 3, 1>(ctx, cls, X, W, w_rows, M, N, K, slices, epi);
     return launch_gemm_tc2p(ctx, cls, X, W, w_rows, M, N, K, epi);
   }
   // token tile: as narrow as the token count allows for weight streaming; 256 where that still gives every SM a CTA pair

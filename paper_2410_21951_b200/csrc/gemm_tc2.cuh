@@ -10,7 +10,9 @@
 // MMAs and signals, through tcgen05.commit to both CTAs, the `empty` barrier of a stage and at the
 // end the accumulator barrier.  TMEM is allocated and freed by warp 1 of both CTAs; the CTAs
 // meet at a cluster barrier after the barrier set-up and before the TMEM is freed.
-// No K split and no LayerNorm operand here; every wait is bounded like in the single-CTA kernel.
+// K is not split over CTAs; with few tokens its slices have an accumulator each, added in order at the end (an accumulation
+// on the tensor cores cuts off where an fp32 addition rounds, so a short chain loses less).  No LayerNorm operand here;
+// every wait is bounded like in the single-CTA kernel.
 #pragma once
 #include "tc.cuh"
 #include "gemm_tc.cuh"
@@ -25,7 +27,6 @@ template <int TN, int ST, int KB> struct GemmTc2Cfg {
   static constexpr int kChunkBytes = kGemmRowsW * kGemmBK * 2 + kXHalfBytes;
   static constexpr int kStageBytes = KB * kChunkBytes;
   static constexpr int kStages = ST;
-  static constexpr int kTmemCols = TN;
   static constexpr int kSmem = kStages * kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
 };
 
@@ -71,7 +72,9 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
 template <int TN, int ST, int KB, typename Epi>
 __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmW,
                                                        const __grid_constant__ CUtensorMap tmX /*box: TN/2 rows*/,
-                                                       int M, int N, int nsteps /*K / (64 KB)*/, Epi epi, uint32_t* err) {
+                                                       int M, int N, int nsteps /*K / (64 KB)*/,
+                                                       int slices /*of K, an accumulator each; divides nsteps*/, Epi epi,
+                                                       uint32_t* err) {
   using Cfg = GemmTc2Cfg<TN, ST, KB>;
   constexpr int S = Cfg::kStages;
   constexpr uint32_t kWBytes = kGemmRowsW * kGemmBK * 2, kXBytes = Cfg::kXHalfBytes;
@@ -94,7 +97,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
     tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmX);
   }
-  if (warp == 1) { tmem_alloc_pair(holder, Cfg::kTmemCols); tmem_relinquish_pair(); }
+  if (warp == 1) { tmem_alloc_pair(holder, TN * slices); tmem_relinquish_pair(); }
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                                    // the peer's barriers exist before anything signals them
@@ -134,8 +137,11 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
     // ---- MMA issuer (leader only): 256 features x TN tokens per instruction
     constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
     grid_dep_wait();                                     // the bounded waits below time this kernel's own pipeline only
-    for (int i = 0; i < nsteps; ++i) {
+    const int per = nsteps / slices;
+    uint32_t acc = tmem;
+    for (int i = 0, left = per; i < nsteps; ++i, --left) {
       const int s = i % S;
+      if (left == 0) { acc += TN; left = per; }
       if (!mbar_wait(full0 + 8 * s, (i / S) & 1, err)) break;
       tc_fence_after();
 #pragma unroll
@@ -143,7 +149,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
         const uint32_t wa = base + s * Cfg::kStageBytes + j * Cfg::kChunkBytes, xa = wa + kWBytes;
 #pragma unroll
         for (int k = 0; k < kGemmBK / 16; ++k)
-          umma_bf16_pair(tmem, umma_desc_k_sw128(wa + 32 * k), umma_desc_k_sw128(xa + 32 * k), idesc, (i | j | k) != 0);
+          umma_bf16_pair(acc, umma_desc_k_sw128(wa + 32 * k), umma_desc_k_sw128(xa + 32 * k), idesc, left != per || (j | k) != 0);
       }
       umma_commit_pair(empty0 + 8 * s);                  // the stage is reusable in both CTAs
     }
@@ -163,13 +169,19 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
     for (int c0 = 0; c0 < TN; c0 += 32) {
       float v[32];
       tmem_ld32(trow + c0, v);
+      for (int u = 1; u < slices; ++u) {                 // the slices of K in order
+        float w[32];
+        tmem_ld32(trow + u * TN + c0, w);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] += w[j];
+      }
       if (n < N && m0 + c0 < M) epi.template col<32>(0, m0 + c0, n, v, M - (m0 + c0));
     }
   }
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                                    // neither CTA frees while the other still reads
-  if (warp == 1) tmem_dealloc_pair(tmem, Cfg::kTmemCols);
+  if (warp == 1) tmem_dealloc_pair(tmem, TN * slices);
 }
 
 }  // namespace vadusa
