@@ -385,8 +385,10 @@ vadusa_status launch_gemm_tc2(vadusa_ctx* ctx, int cls, const void* X, const voi
   static unsigned long long attr_done = 0ull;              // per device, like launch_gemm_tc
   const unsigned long long dev_bit = 1ull << (ctx->cfg.device & 63);
   if (!(attr_done & dev_bit)) {
-    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
-    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, Epi>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, false, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
+    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, true, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmem));
+    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, false, Epi>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+    CU(cudaFuncSetAttribute(gemm_tc2_kernel<TN, ST, KB, true, Epi>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     attr_done |= dev_bit;
   }
   const CUtensorMap *mw, *mx;
@@ -404,7 +406,7 @@ vadusa_status launch_gemm_tc2(vadusa_ctx* ctx, int cls, const void* X, const voi
   at[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at; lc.numAttrs = 2;
   PROF(ctx, cls);
-  CU(cudaLaunchKernelEx(&lc, gemm_tc2_kernel<TN, ST, KB, Epi>, *mw, *mx, M, N, K / (kGemmBK * KB), slices, epi, err_word(ctx)));
+  CU(cudaLaunchKernelEx(&lc, slices > 1 ? gemm_tc2_kernel<TN, ST, KB, true, Epi> : gemm_tc2_kernel<TN, ST, KB, false, Epi>, *mw, *mx, M, N, K / (kGemmBK * KB), slices, epi, err_word(ctx)));
   LAUNCH_CHECK();
   return VADUSA_OK;
 }
@@ -496,7 +498,7 @@ vadusa_status gemm_tc(vadusa_ctx* ctx, int cls, const void* X, const void* W, in
     auto ctas = [&](int tn) { return ntiles_n * ((M + tn - 1) / tn); };
     // Accumulators: one; for a prefix, whose rows every later token reads, one per K slice that a single-CTA product of 128-token
     // tiles would be split into (shorter chains of truncating additions: the rows are the split form's to the bit).  One prefix
-    // of 325 tokens 668 -> 726 us a call; the same in a batch-8 step would be 3.00 -> 3.19 ms.
+    // of 325 tokens 668 -> 713 us a call; the same in a batch-8 step would be 3.00 -> 3.19 ms.
     const int slices = !ctx->in_prefill || (M > 512 && ctas(128) >= 128) ? 1 : gemm_ksplit(ctas(128), K / kGemmBK, 128);
     const bool two = K % (2 * kGemmBK) == 0;             // stages of two chunks
     if (two && ctas(32) <= (N <= K ? 148 : 72)) {

@@ -69,7 +69,7 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
                ::"r"(bar), "h"(both) : "memory");
 }
 
-template <int TN, int ST, int KB, typename Epi>
+template <int TN, int ST, int KB, bool SL /*more than one slice*/, typename Epi>
 __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmW,
                                                        const __grid_constant__ CUtensorMap tmX /*box: TN/2 rows*/,
                                                        int M, int N, int nsteps /*K / (64 KB)*/,
@@ -137,11 +137,12 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
     // ---- MMA issuer (leader only): 256 features x TN tokens per instruction
     constexpr uint32_t idesc = umma_idesc_bf16(2 * kGemmRowsW, TN);
     grid_dep_wait();                                     // the bounded waits below time this kernel's own pipeline only
+    if (!SL) slices = 1;
     const int per = nsteps / slices;
     uint32_t acc = tmem;
     for (int i = 0, left = per; i < nsteps; ++i, --left) {
       const int s = i % S;
-      if (left == 0) { acc += TN; left = per; }
+      if (SL && left == 0) { acc += TN; left = per; }
       if (!mbar_wait(full0 + 8 * s, (i / S) & 1, err)) break;
       tc_fence_after();
 #pragma unroll
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
         const uint32_t wa = base + s * Cfg::kStageBytes + j * Cfg::kChunkBytes, xa = wa + kWBytes;
 #pragma unroll
         for (int k = 0; k < kGemmBK / 16; ++k)
-          umma_bf16_pair(acc, umma_desc_k_sw128(wa + 32 * k), umma_desc_k_sw128(xa + 32 * k), idesc, left != per || (j | k) != 0);
+          umma_bf16_pair(acc, umma_desc_k_sw128(wa + 32 * k), umma_desc_k_sw128(xa + 32 * k), idesc, (SL ? left != per : i != 0) || (j | k) != 0);
       }
       umma_commit_pair(empty0 + 8 * s);                  // the stage is reusable in both CTAs
     }
@@ -169,7 +170,8 @@ __global__ void __launch_bounds__(128) gemm_tc2_kernel(const __grid_constant__ C
     for (int c0 = 0; c0 < TN; c0 += 32) {
       float v[32];
       tmem_ld32(trow + c0, v);
-      for (int u = 1; u < slices; ++u) {                 // the slices of K in order
+#pragma unroll 1
+      for (int u = 1; SL && u < slices; ++u) {                 // the slices of K in order
         float w[32];
         tmem_ld32(trow + u * TN + c0, w);
 #pragma unroll
